@@ -13,11 +13,14 @@
 #define STAGE_THREADS 128
 #define STAGE_STRIDE 129
 
-// i: the thread's index inside its 128-thread staging unit (a multiple of 32 apart from
-// threadIdx.x, so the warp-level ballots below see the same lanes)
+// i: the thread's index inside its staging unit of 128 threads, or of one warp (two groups); a multiple
+// of 32 apart from threadIdx.x, so the warp-level ballots below see the same lanes. STRIDE: words between
+// texel rows, one more than the unit's blocks. STEPS: steps of four coefficients unrolled (4: all loads in
+// flight together; 1: a quarter of the code).
+template <int STRIDE, int STEPS = 4>
 __device__ __forceinline__ void stage_groups(const float* __restrict__ sh, const int32_t* __restrict__ perm,
                                              const float* s_scale, int64_t g0, int64_t n_groups,
-                                             uint32_t (*tex)[STAGE_STRIDE], int i) {
+                                             uint32_t (*tex)[STRIDE], int i) {
   const int lg = i >> 4, t = i & 15;
   const int64_t g = g0 + lg;
   const bool live = g < n_groups;
@@ -36,17 +39,17 @@ __device__ __forceinline__ void stage_groups(const float* __restrict__ sh, const
     return;
   }
   const float4* p = reinterpret_cast<const float4*>(sh + (int64_t)src * 48);
-  float v[48];
+  // four coefficients (three 16-byte loads) per step
+#pragma unroll STEPS
+  for (int j = 0; j < 4; j++) {
+    const float4 a = __ldg(p + 3 * j), b = __ldg(p + 3 * j + 1), c = __ldg(p + 3 * j + 2);
+    const float v[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
 #pragma unroll
-  for (int j = 0; j < 12; j++) {
-    float4 f = __ldg(p + j);
-    v[4 * j + 0] = f.x; v[4 * j + 1] = f.y; v[4 * j + 2] = f.z; v[4 * j + 3] = f.w;
-  }
-#pragma unroll
-  for (int k = 0; k < 16; k++) {
-    float s = s_scale[k];
-    uint32_t r = gsc_quant1(v[3 * k + 0], s), gg = gsc_quant1(v[3 * k + 1], s), b = gsc_quant1(v[3 * k + 2], s);
-    tex[t][col + k] = r | (gg << 8) | (b << 16);
+    for (int k = 0; k < 4; k++) {
+      const float s = s_scale[4 * j + k];
+      const uint32_t r = gsc_quant1(v[3 * k + 0], s), g = gsc_quant1(v[3 * k + 1], s), b8 = gsc_quant1(v[3 * k + 2], s);
+      tex[t][col + 4 * j + k] = r | (g << 8) | (b8 << 16);
+    }
   }
 }
 
