@@ -13,7 +13,7 @@ LIB = os.path.join(PKG, "lib", "libgsc.so")
 # the checked build: slot-order entries bounds-checked in the decoders (GSC_CHECKED)
 BUILD_CHECKED = os.path.join(PKG, "_build_checked")
 LIB_CHECKED = os.path.join(PKG, "lib", "libgsc_checked.so")
-SOURCES = ["api.cu", "plan.cu", "bc1.cu", "bc7.cu", "rate.cu", "decode.cu", "layout.cu", "render.cu",
+SOURCES = ["api.cu", "plan.cu", "sort.cu", "bc1.cu", "bc7.cu", "rate.cu", "decode.cu", "layout.cu", "render.cu",
            "geometry.cu", "batch.cu", "serve.cu", "scene_file.cu", "shard.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

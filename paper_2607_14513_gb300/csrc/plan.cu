@@ -1,201 +1,10 @@
 // plan.cu -- per-scene scales, quantisation and the reorder plan (Sec. V-A; Sec. III-C,
-// Fig. Bit4Scan), plus the device-wide radix sort and scan the plan and the rate
-// control share. No host synchronisation: everything is queued on the caller's stream.
+// Fig. Bit4Scan). No host synchronisation: everything is queued on the caller's stream.
 #include <mutex>
 
-#include "gsc_internal.cuh"
+#include "sort.cuh"
 
-// ---- scan (exclusive, 64-bit) -------------------------------------------------------------
-#define SCAN_BLOCK 1024
-static int64_t scan_blocks(int64_t n) { return ceil_div64(n > 0 ? n : 1, SCAN_BLOCK); }
-size_t scan_ws_bytes(int64_t n) {
-  int64_t nb = scan_blocks(n);
-  return align_up(sizeof(uint64_t) * (size_t)nb, 256) + align_up(sizeof(uint64_t) * (size_t)scan_blocks(nb), 256) + 256;
-}
-
-template <class T>
-__device__ __forceinline__ uint64_t block_excl_scan(uint64_t v, uint64_t* s_warp, uint64_t* total) {
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  uint64_t x = v;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    uint64_t y = __shfl_up_sync(0xFFFFFFFFu, x, d);
-    if (lane >= d) x += y;
-  }
-  if (lane == 31) s_warp[w] = x;
-  __syncthreads();
-  if (w == 0) {
-    uint64_t y = lane < (int)(blockDim.x >> 5) ? s_warp[lane] : 0;
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      uint64_t z = __shfl_up_sync(0xFFFFFFFFu, y, d);
-      if (lane >= d) y += z;
-    }
-    s_warp[lane] = y;  // inclusive over warps
-  }
-  __syncthreads();
-  uint64_t before = (w > 0 ? s_warp[w - 1] : 0) + x - v;
-  if (total) *total = s_warp[(blockDim.x >> 5) - 1];
-  __syncthreads();
-  return before;
-}
-
-template <class T>
-__global__ void k_scan_reduce(const T* __restrict__ in, int64_t n, uint64_t* __restrict__ sums) {
-  __shared__ uint64_t s_warp[32];
-  const int64_t i = (int64_t)blockIdx.x * SCAN_BLOCK + threadIdx.x;
-  uint64_t v = i < n ? (uint64_t)in[i] : 0;
-  uint64_t tot;
-  block_excl_scan<T>(v, s_warp, &tot);
-  if (threadIdx.x == 0) sums[blockIdx.x] = tot;
-}
-
-template <class T>
-__global__ void k_scan_apply(const T* __restrict__ in, int64_t n, const uint64_t* __restrict__ offs,
-                             T* __restrict__ out, uint64_t* __restrict__ total) {
-  __shared__ uint64_t s_warp[32];
-  const int64_t i = (int64_t)blockIdx.x * SCAN_BLOCK + threadIdx.x;
-  uint64_t v = i < n ? (uint64_t)in[i] : 0;
-  uint64_t tot;
-  uint64_t ex = block_excl_scan<T>(v, s_warp, &tot) + (offs ? offs[blockIdx.x] : 0);
-  if (i < n) out[i] = (T)ex;
-  if (total && blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) *total = (offs ? offs[blockIdx.x] : 0) + tot;
-}
-
-// single-block scan of up to SCAN_BLOCK * k elements held in one array (sequential chunks)
-__global__ void k_scan_single(uint64_t* __restrict__ a, int64_t n) {
-  __shared__ uint64_t s_warp[32];
-  __shared__ uint64_t carry;
-  if (threadIdx.x == 0) carry = 0;
-  __syncthreads();
-  for (int64_t base = 0; base < n; base += SCAN_BLOCK) {
-    const int64_t i = base + threadIdx.x;
-    uint64_t v = i < n ? a[i] : 0;
-    uint64_t tot;
-    uint64_t ex = block_excl_scan<uint64_t>(v, s_warp, &tot);
-    if (i < n) a[i] = ex + carry;
-    __syncthreads();
-    if (threadIdx.x == 0) carry += tot;
-    __syncthreads();
-  }
-}
-
-// Exclusive scan of n values of T (uint32 or uint64) into out (may alias in); total (device, optional).
-template <class T>
-cudaError_t scan_exclusive(const T* in, T* out, int64_t n, uint64_t* total, void* ws, cudaStream_t st) {
-  if (n <= 0) return cudaSuccess;
-  int64_t nb = scan_blocks(n);
-  uint64_t* sums = reinterpret_cast<uint64_t*>(ws);
-  gsc_count_launch(); k_scan_reduce<T><<<(int)nb, SCAN_BLOCK, 0, st>>>(in, n, sums);
-  gsc_count_launch(); k_scan_single<<<1, SCAN_BLOCK, 0, st>>>(sums, nb);
-  gsc_count_launch(); k_scan_apply<T><<<(int)nb, SCAN_BLOCK, 0, st>>>(in, n, sums, out, total);
-  return cudaGetLastError();
-}
-template cudaError_t scan_exclusive<uint32_t>(const uint32_t*, uint32_t*, int64_t, uint64_t*, void*, cudaStream_t);
-template cudaError_t scan_exclusive<uint64_t>(const uint64_t*, uint64_t*, int64_t, uint64_t*, void*, cudaStream_t);
-
-// ---- stable LSD radix sort of (u64 key, u32 value) pairs, 8-bit digits ---------------------
-#define RS_THREADS 256
-#define RS_ITEMS 8
-#define RS_TILE (RS_THREADS * RS_ITEMS)
-
-static int64_t rs_tiles(int64_t n) { return ceil_div64(n > 0 ? n : 1, RS_TILE); }
-
-size_t radix_ws_bytes(int64_t n) {
-  int64_t nt = rs_tiles(n);
-  size_t b = 0;
-  b += align_up(sizeof(uint64_t) * (size_t)(n > 0 ? n : 1), 256);   // keys ping-pong
-  b += align_up(sizeof(uint32_t) * (size_t)(n > 0 ? n : 1), 256);   // values ping-pong
-  b += align_up(sizeof(uint32_t) * 256 * (size_t)nt, 256);          // digit x tile counts
-  b += scan_ws_bytes(256 * nt);
-  return b + 1024;
-}
-
-__global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const uint64_t* __restrict__ keys, int64_t n, int shift,
-                                                       uint32_t* __restrict__ hist, int64_t n_tiles) {
-  __shared__ uint32_t h[256];
-  h[threadIdx.x] = 0;
-  __syncthreads();
-  const int64_t base = (int64_t)blockIdx.x * RS_TILE;
-#pragma unroll
-  for (int r = 0; r < RS_ITEMS; r++) {
-    int64_t i = base + r * RS_THREADS + threadIdx.x;
-    if (i < n) atomicAdd(&h[(keys[i] >> shift) & 255], 1u);
-  }
-  __syncthreads();
-  hist[(int64_t)threadIdx.x * n_tiles + blockIdx.x] = h[threadIdx.x];
-}
-
-__global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint64_t* __restrict__ kin,
-                                                          const uint32_t* __restrict__ vin, int64_t n, int shift,
-                                                          const uint32_t* __restrict__ offs, int64_t n_tiles,
-                                                          uint64_t* __restrict__ kout, uint32_t* __restrict__ vout) {
-  __shared__ uint32_t run[256];
-  __shared__ uint16_t wcnt[RS_THREADS / 32][256];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  run[threadIdx.x] = 0;
-  const int64_t base = (int64_t)blockIdx.x * RS_TILE;
-  const uint32_t lt = (1u << lane) - 1u;
-  for (int r = 0; r < RS_ITEMS; r++) {
-    const int64_t i = base + r * RS_THREADS + threadIdx.x;
-    const bool live = i < n;
-    uint64_t k = live ? kin[i] : 0;
-    uint32_t v = live ? vin[i] : 0;
-    const uint32_t d = live ? (uint32_t)((k >> shift) & 255) : 256u;
-#pragma unroll
-    for (int q = 0; q < 8; q++) wcnt[w][lane * 8 + q] = 0;
-    __syncwarp();
-    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, d);
-    const int leader = __ffs(peers) - 1;
-    if (live && lane == leader) wcnt[w][d] = (uint16_t)__popc(peers);
-    __syncthreads();
-    if (live) {
-      uint32_t pos = run[d] + __popc(peers & lt);
-      for (int ww = 0; ww < w; ww++) pos += wcnt[ww][d];
-      const uint32_t dst = offs[(int64_t)d * n_tiles + blockIdx.x] + pos;
-      kout[dst] = k;
-      vout[dst] = v;
-    }
-    __syncthreads();
-    uint32_t add = 0;
-#pragma unroll
-    for (int ww = 0; ww < RS_THREADS / 32; ww++) add += wcnt[ww][threadIdx.x];
-    run[threadIdx.x] += add;
-    __syncthreads();
-  }
-}
-
-cudaError_t radix_sort_pairs(uint64_t* keys, uint32_t* vals, int64_t n, int key_bits, void* ws, cudaStream_t st) {
-  if (n <= 1 || key_bits <= 0) return cudaSuccess;
-  const int64_t nt = rs_tiles(n);
-  Carve c{reinterpret_cast<uint8_t*>(ws), 0, 0};
-  uint64_t* k2 = c.take<uint64_t>(n);
-  uint32_t* v2 = c.take<uint32_t>(n);
-  uint32_t* hist = c.take<uint32_t>(256 * nt);
-  void* sws = c.take<uint8_t>((int64_t)scan_ws_bytes(256 * nt));
-  uint64_t* ka = keys;
-  uint32_t* va = vals;
-  uint64_t* kb = k2;
-  uint32_t* vb = v2;
-  int passes = (key_bits + 7) / 8;
-  for (int p = 0; p < passes; p++) {
-    gsc_count_launch(); k_rs_hist<<<(int)nt, RS_THREADS, 0, st>>>(ka, n, 8 * p, hist, nt);
-    cudaError_t e = scan_exclusive<uint32_t>(hist, hist, 256 * nt, nullptr, sws, st);
-    if (e != cudaSuccess) return e;
-    gsc_count_launch(); k_rs_scatter<<<(int)nt, RS_THREADS, 0, st>>>(ka, va, n, 8 * p, hist, nt, kb, vb);
-    uint64_t* tk = ka; ka = kb; kb = tk;
-    uint32_t* tv = va; va = vb; vb = tv;
-  }
-  if (ka != keys) {
-    cudaError_t e = cudaMemcpyAsync(keys, ka, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return e;
-    e = cudaMemcpyAsync(vals, va, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, st);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaGetLastError();
-}
-
-// ---- scales: exact order statistic by 4 passes of 8-bit radix select -----------------------
+// ---- scales of a sharded scene: exact order statistic by 4 passes of 8-bit radix select --------
 struct SelState { uint32_t prefix[GSC_SH]; uint64_t rank[GSC_SH]; };
 
 __global__ void k_sel_init(SelState* s, uint64_t r) {
@@ -432,12 +241,12 @@ gsc_status plan_run(gsc_ctx* ctx, const float* pos, const float* sh, const gsc_p
   gsc_count_launch(); k_bbox<<<grid_stride(n, 256, ctx->sm_count * 2), 256, 0, st>>>(pos, n, bb);
   gsc_count_launch(); k_morton<<<grid_stride(n, 256), 256, 0, st>>>(pos, n, bb, keys, vals);
   GSC_CUDA(cudaGetLastError());
-  GSC_CUDA(radix_sort_pairs(keys, vals, n, 30, rws, st));
+  GSC_CUDA(radix_sort_pairs(keys, vals, n, 30, rws, ctx->d_status, st));
   // slot order: stable sort by (chunk, colour key) of the rank-ordered Gaussians
   gsc_count_launch(); k_colour_keys<<<grid_stride(n, 256), 256, 0, st>>>(sh, scales, n, pp->group_size, keys, vals);
   GSC_CUDA(cudaGetLastError());
   const uint64_t max_chunk = pp->group_size ? (uint64_t)((n - 1) / pp->group_size) : 0;
-  GSC_CUDA(radix_sort_pairs(keys, vals, n, 24 + bits_for(max_chunk), rws, st));
+  GSC_CUDA(radix_sort_pairs(keys, vals, n, 24 + bits_for(max_chunk), rws, ctx->d_status, st));
   gsc_count_launch(); k_finish_perm<<<grid_stride(ns, 256), 256, 0, st>>>(vals, n, ns, 0, perm);
   GSC_CUDA(cudaGetLastError());
   return GSC_OK;
@@ -539,13 +348,13 @@ cudaError_t shard_morton(const float* pos, int64_t n, const int64_t* bb, uint64_
 
 size_t shard_order_ws_bytes(int64_t n) { return radix_ws_bytes(n) + 256; }
 
-cudaError_t shard_order(uint64_t* keys, int64_t n, int32_t* order, void* ws, int sm_count, cudaStream_t st) {
+cudaError_t shard_order(uint64_t* keys, int64_t n, int32_t* order, void* ws, int sm_count, int* err, cudaStream_t st) {
   if (n == 0) return cudaSuccess;
   uint32_t* vals = reinterpret_cast<uint32_t*>(order);
   gsc_count_launch(); k_iota<<<grid_stride(n, 256, sm_count * 8), 256, 0, st>>>(vals, n);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  return radix_sort_pairs(keys, vals, n, 30, ws, st);  // stable: equal codes keep the input order
+  return radix_sort_pairs(keys, vals, n, 30, ws, err, st);  // stable: equal codes keep the input order
 }
 
 size_t shard_select_state_bytes() { return align_up(sizeof(SelState), 256) + sizeof(uint32_t) * GSC_SH * 256; }
@@ -593,7 +402,7 @@ size_t shard_plan_ws_bytes(int64_t n) {
 // Slot order of a shard whose Gaussians are given in spatial-rank order and whose first one
 // starts a chunk: the stable (chunk, colour key) sort of the whole-scene plan, on this range.
 gsc_status shard_plan(const float* sh, int64_t n, const float* scales, int64_t group_size, int32_t* perm, void* ws,
-                      size_t ws_bytes, int sm_count, cudaStream_t st) {
+                      size_t ws_bytes, int sm_count, int* err, cudaStream_t st) {
   const int64_t ns = ceil_div64(n, 16) * 16;
   if (ws_bytes < shard_plan_ws_bytes(n)) return GSC_ERR_OOM;
   if (ns == 0) return GSC_OK;
@@ -605,7 +414,7 @@ gsc_status shard_plan(const float* sh, int64_t n, const float* scales, int64_t g
   gsc_count_launch(); k_colour_keys<<<grid_stride(n, 256, sm_count * 8), 256, 0, st>>>(sh, scales, n, group_size, keys, vals);
   GSC_CUDA(cudaGetLastError());
   const uint64_t max_chunk = (uint64_t)((n - 1) / group_size);
-  GSC_CUDA(radix_sort_pairs(keys, vals, n, 24 + bits_for(max_chunk), rws, st));
+  GSC_CUDA(radix_sort_pairs(keys, vals, n, 24 + bits_for(max_chunk), rws, err, st));
   gsc_count_launch(); k_finish_perm<<<grid_stride(ns, 256, sm_count * 8), 256, 0, st>>>(vals, n, ns, 0, perm);
   GSC_CUDA(cudaGetLastError());
   return GSC_OK;
