@@ -102,6 +102,7 @@ gsc_status ctx_new(int device, bool init_tables, gsc_ctx** out);
 
 // ---- launchers implemented by the translation units ------------------------------
 // plan.cu
+cudaError_t plan_init();
 size_t plan_ws_bytes(int64_t n);
 gsc_status plan_run(gsc_ctx* ctx, const float* pos, const float* sh, const gsc_plan_params* pp, int32_t* perm,
                     float* scales, void* ws, size_t ws_bytes, cudaStream_t st);
@@ -114,15 +115,14 @@ template <class T>
 cudaError_t scan_exclusive(const T* in, T* out, int64_t n, uint64_t* total, void* ws, cudaStream_t st);
 // Stable LSD radix sort of n (key, 32-bit value) pairs, K uint32_t or uint64_t, on the low key_bits bits, between the
 // caller's two pairs of arrays; *out_keys / *out_vals: where the result is. iota: the values are the input positions
-// (vals is not read); want_keys = false: the sorted keys may be left unwritten. state: radix_state_bytes(n), 256-byte
-// aligned. err (optional): a context's status word, which gets GSC_ERR_TIMEOUT if a bounded device wait gives up.
+// (vals is not read); want_keys = false: the sorted keys may be left unwritten. state: radix_state_bytes(n).
 size_t radix_state_bytes(int64_t n);
 template <class K>
-cudaError_t radix_sort(K* keys, K* keys2, uint32_t* vals, uint32_t* vals2, int64_t n, int key_bits, bool iota,
-                       bool want_keys, void* state, int* err, cudaStream_t st, K** out_keys, uint32_t** out_vals);
+cudaError_t radix_sort(K* keys, K* keys2, uint32_t* vals, uint32_t* vals2, int64_t n, int key_bits, bool iota, bool want_keys,
+                       void* state, cudaStream_t st, K** out_keys, uint32_t** out_vals);
 // The same for 64-bit keys with the result in keys / vals; ws (radix_ws_bytes) holds the second arrays and the state.
 size_t radix_ws_bytes(int64_t n);
-cudaError_t radix_sort_pairs(uint64_t* keys, uint32_t* vals, int64_t n, int key_bits, void* ws, int* err, cudaStream_t st);
+cudaError_t radix_sort_pairs(uint64_t* keys, uint32_t* vals, int64_t n, int key_bits, void* ws, cudaStream_t st);
 
 // bc1.cu
 cudaError_t bc1_init_tables();
@@ -209,7 +209,7 @@ gsc_status decode_blocks_tex_run(gsc_ctx* ctx, const uint8_t* blocks, int64_t nb
 cudaError_t shard_bbox(const float* pos, int64_t n, int64_t* bb, int sm_count, cudaStream_t st);
 cudaError_t shard_morton(const float* pos, int64_t n, const int64_t* bb, uint64_t* keys, int sm_count, cudaStream_t st);
 size_t shard_order_ws_bytes(int64_t n);
-cudaError_t shard_order(uint64_t* keys, int64_t n, int32_t* order, void* ws, int sm_count, int* err, cudaStream_t st);
+cudaError_t shard_order(uint64_t* keys, int64_t n, int32_t* order, void* ws, int sm_count, cudaStream_t st);
 size_t shard_select_state_bytes();
 cudaError_t shard_select_begin(int64_t n_total, int permille, void* state, cudaStream_t st);
 cudaError_t shard_select_hist(const float* sh, int64_t n, int shift, void* state, int64_t* hist, int sm_count,
@@ -218,7 +218,7 @@ cudaError_t shard_select_pick(void* state, const int64_t* hist_total, int shift,
 cudaError_t shard_select_scales(const void* state, float* scales, cudaStream_t st);
 size_t shard_plan_ws_bytes(int64_t n);
 gsc_status shard_plan(const float* sh, int64_t n, const float* scales, int64_t group_size, int32_t* perm, void* ws,
-                      size_t ws_bytes, int sm_count, int* err, cudaStream_t st);
+                      size_t ws_bytes, int sm_count, cudaStream_t st);
 size_t shard_rate_ws_bytes(int64_t ng);
 gsc_status shard_rate_begin(gsc_ctx* ctx, const float* sh, int64_t n, const int32_t* perm, const float* scales,
                             uint8_t* b1, uint8_t* b7, void* ws, size_t ws_bytes, int64_t* part, cudaStream_t st);

@@ -327,7 +327,7 @@ gsc_status rate_select(gsc_ctx* ctx, int64_t n, const int32_t* perm, const float
   gsc_count_launch(); k_fill_apply<<<gsz(ng, 256, cap), 256, 0, st>>>(ng, S, mode, alt, delta, prefix, keys, vals);
   gsc_count_launch(); k_stream_info<<<1, 32, 0, st>>>(S, w, info);
   GSC_CUDA(cudaGetLastError());
-  GSC_CUDA(radix_sort_pairs(keys, vals, ng, 4, rws, ctx->d_status, st));
+  GSC_CUDA(radix_sort_pairs(keys, vals, ng, 4, rws, st));
   gsc_count_launch(); k_assemble<<<gsz(ng, 128, cap), 128, 0, st>>>(keys, vals, ng, info, reinterpret_cast<const uint2*>(b1),
                                                  reinterpret_cast<const uint2*>(b7), perm, blocks, perm_out);
   GSC_CUDA(cudaGetLastError());
@@ -635,7 +635,7 @@ gsc_status shard_rate_assemble(gsc_ctx* ctx, int64_t ng, void* ws, const uint8_t
   gsc_count_launch(); k_shard_info<<<1, 32, 0, st>>>(r.S, r.w, counts_all, n_shards, shard, r.info);
   GSC_CUDA(cudaGetLastError());
   if (ng > 0) {
-    GSC_CUDA(radix_sort_pairs(r.keys, r.vals, ng, 4, r.rws, ctx->d_status, st));
+    GSC_CUDA(radix_sort_pairs(r.keys, r.vals, ng, 4, r.rws, st));
     gsc_count_launch();
     k_shard_assemble<<<gsz(ng, 128, ctx->sm_count * 8), 128, 0, st>>>(
         r.keys, r.vals, ng, r.info, reinterpret_cast<const uint2*>(b1), reinterpret_cast<const uint2*>(b7), perm,

@@ -505,7 +505,7 @@ gsc_status render_run(gsc_ctx* c, const DevTable& T, const uint8_t* d_blocks, co
     gsc_count_launch();
     k_depth_keys<<<grid_of(n), 256, 0, st>>>(n, w.rec, w.count, w.dkey, w.dval);
     GSC_CUDA(cudaGetLastError());
-    GSC_CUDA(radix_sort_pairs(w.dkey, w.dval, n, 32, w.radix_ws, c->d_status, st));
+    GSC_CUDA(radix_sort_pairs(w.dkey, w.dval, n, 32, w.radix_ws, st));
     gsc_count_launch();
     k_gather_counts<<<grid_of(n), 256, 0, st>>>(n, w.dval, w.count, w.count_sorted);
     GSC_CUDA(cudaGetLastError());
@@ -524,7 +524,7 @@ gsc_status render_run(gsc_ctx* c, const DevTable& T, const uint8_t* d_blocks, co
     k_splat_keys<<<grid_of(n), 256, 0, st>>>(n, w.dval, w.rect, w.count_sorted, w.offset, cd.tiles_x, w.keys,
                                              w.vals);
     GSC_CUDA(cudaGetLastError());
-    GSC_CUDA(radix_sort_pairs(w.keys, w.vals, (int64_t)pairs, tile_bits(tiles), w.radix_ws, c->d_status, st));
+    GSC_CUDA(radix_sort_pairs(w.keys, w.vals, (int64_t)pairs, tile_bits(tiles), w.radix_ws, st));
     gsc_count_launch();
     k_tile_ranges<<<grid_of((int64_t)pairs), 256, 0, st>>>(w.keys, (int64_t)pairs, w.ranges);
     GSC_CUDA(cudaGetLastError());

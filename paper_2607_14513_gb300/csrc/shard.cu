@@ -53,7 +53,7 @@ extern "C" gsc_status gsc_shard_order(gsc_ctx* c, uint64_t* d_keys, int64_t n_to
   if (!al(d_keys, 8) || !al(d_order, 4) || !al(d_ws, 256)) return GSC_ERR_INVALID_ARG;
   if (n_total > 0 && ws_bytes < shard_order_ws_bytes(n_total)) return GSC_ERR_OOM;
   GSC_CUDA(cudaSetDevice(c->device));
-  GSC_CUDA(shard_order(d_keys, n_total, d_order, d_ws, c->sm_count, c->d_status, (cudaStream_t)stream));
+  GSC_CUDA(shard_order(d_keys, n_total, d_order, d_ws, c->sm_count, (cudaStream_t)stream));
   return GSC_OK;
 }
 
@@ -104,7 +104,7 @@ extern "C" gsc_status gsc_shard_plan(gsc_ctx* c, const float* d_sh, int64_t n, c
   if (!al(d_sh, 16) || !al(d_perm, 4) || !al(d_ws, 256)) return GSC_ERR_INVALID_ARG;
   GSC_CUDA(cudaSetDevice(c->device));
   GscTimed tm(c, T_PLAN, (cudaStream_t)stream);
-  return shard_plan(d_sh, n, d_scales, group_size, d_perm, d_ws, ws_bytes, c->sm_count, c->d_status, (cudaStream_t)stream);
+  return shard_plan(d_sh, n, d_scales, group_size, d_perm, d_ws, ws_bytes, c->sm_count, (cudaStream_t)stream);
 }
 
 static bool rate_ws_ok(int64_t n, const void* d_ws) { return n_ok(n) && d_ws && al(d_ws, 256); }

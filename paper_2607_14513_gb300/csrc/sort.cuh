@@ -23,30 +23,32 @@ __device__ __forceinline__ uint64_t prefix256(uint64_t v, uint64_t* s) {
 }
 
 // Stable ranks of a CTA's items by an 8-bit digit. Warp w holds ITEMS * 32 consecutive items, item r of lane l
-// being r * 32 + l of them; digit[r] = 256 for an item past the end. On return rank[r] is the item's position
+// being r * 32 + l of them; digit(r) = 256 for an item past the end. On return rank[r] is the item's position
 // among its warp's items of the same digit, and cnt[w][d] the number of items of digit d in the warps before w;
-// the total per digit is returned to thread d < 256. cnt has WARPS rows. Each round's peers are found with one
-// match; the warp's counters are its own, so rounds need no CTA barrier.
-template <int WARPS, int ITEMS>
-__device__ __forceinline__ uint32_t rank_digits(const uint32_t (&digit)[ITEMS], uint32_t (&rank)[ITEMS],
-                                                uint16_t (*cnt)[256]) {
+// the total per digit is returned to thread d < 256. cnt has WARPS rows. A round's peers come from eight ballots
+// (a match instruction took several times as long on digits that mostly differ), and its leaders take their
+// places with one shared-memory addition each: rounds wait neither for one another nor for a barrier.
+template <int WARPS, int ITEMS, class Digit>
+__device__ __forceinline__ uint32_t rank_digits(Digit digit, uint32_t (&rank)[ITEMS], uint32_t (*cnt)[256]) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t below = (1u << lane) - 1u;
-  {
-    uint32_t* z = reinterpret_cast<uint32_t*>(cnt[w]);
 #pragma unroll
-    for (int q = 0; q < 4; q++) z[lane + 32 * q] = 0u;
-  }
+  for (int q = 0; q < 8; q++) cnt[w][lane + 32 * q] = 0u;
   __syncwarp();
 #pragma unroll
   for (int r = 0; r < ITEMS; r++) {
-    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, digit[r]);
+    const uint32_t d = digit(r);
+    const bool live = d < 256u;
+    uint32_t peers = __ballot_sync(0xFFFFFFFFu, live);
+#pragma unroll
+    for (int b = 0; b < 8; b++) {
+      const uint32_t set = __ballot_sync(0xFFFFFFFFu, (d >> b) & 1u);
+      peers &= (d >> b) & 1u ? set : ~set;
+    }
     const uint32_t before = __popc(peers & below);
-    const uint32_t old = digit[r] < 256u ? cnt[w][digit[r]] : 0u;
-    rank[r] = old + before;
-    __syncwarp();
-    if (digit[r] < 256u && before == 0u) cnt[w][digit[r]] = (uint16_t)(old + __popc(peers));
-    __syncwarp();
+    uint32_t old = 0u;
+    if (live && before == 0u) old = atomicAdd(&cnt[w][d], (uint32_t)__popc(peers));
+    rank[r] = __shfl_sync(0xFFFFFFFFu, old, live ? __ffs(peers) - 1 : lane) + before;
   }
   __syncthreads();
   uint32_t sum = 0;
@@ -54,7 +56,7 @@ __device__ __forceinline__ uint32_t rank_digits(const uint32_t (&digit)[ITEMS], 
 #pragma unroll
     for (int k = 0; k < WARPS; k++) {
       const uint32_t c = cnt[k][threadIdx.x];
-      cnt[k][threadIdx.x] = (uint16_t)sum;
+      cnt[k][threadIdx.x] = sum;
       sum += c;
     }
   }
