@@ -113,7 +113,7 @@ size_t scan_ws_bytes(int64_t n);
 // Exclusive scan of n values (uint32 or uint64); *total (device, optional) gets the sum.
 template <class T>
 cudaError_t scan_exclusive(const T* in, T* out, int64_t n, uint64_t* total, void* ws, cudaStream_t st);
-// Stable LSD radix sort of n (key, 32-bit value) pairs, K uint32_t or uint64_t, on the low key_bits bits, between the
+// Stable LSD radix sort of n (key, 32-bit value) pairs, K uint16_t, uint32_t or uint64_t, on the low key_bits bits, between the
 // caller's two pairs of arrays; *out_keys / *out_vals: where the result is. iota: the values are the input positions
 // (vals is not read); want_keys = false: the sorted keys may be left unwritten. state: radix_state_bytes(n).
 size_t radix_state_bytes(int64_t n);

@@ -7,8 +7,8 @@
 // depth, 2-D covariance with a 0.3 px^2 low-pass, its inverse, the 3-sigma square's 16 x 16 tile
 // rectangle, mu = sigmoid(t)); a stable radix sort of the visible Gaussians by depth; a scan of
 // their tile counts in that order; one tile key per overlapped tile, emitted in depth order; a
-// stable radix sort by tile (each tile's list stays nearest first); tile ranges; and one CTA per
-// tile blending its list front to back, two pixels per thread. The setup's decisions (culling, rectangle, depth order) are taken in
+// stable radix sort by tile (each tile's list stays nearest first); tile ranges; and one warp per
+// tile blending its list front to back, eight pixels per thread. The setup's decisions (culling, rectangle, depth order) are taken in
 // float with a fixed order of correctly rounded operations, so every implementation of the same
 // steps takes them the same way.
 #include <math.h>
@@ -35,13 +35,15 @@ __device__ __forceinline__ float dot3(float a0, float b0, float a1, float b1, fl
   return fa(fa(fm(a0, b0), fm(a1, b1)), fm(a2, b2));
 }
 
-// Splat of Gaussian i (Eq. covar, the EWA projection, its tile rectangle): rec0 = (u, v, mu,
-// depth), rec1 = conic scaled for exp2, rec2 = premultiplied colour; rect = tile rectangle [x0, x1)
-// x [y0, y1). Returns its tile count (0: culled).
+// Splat of Gaussian i (Eq. covar, the EWA projection, its tile rectangle): rec0 = (u, v, k0, k1),
+// rec1 = (k2, -mu, r, g), rec2.x = b with the exponent k0 dx^2 + k1 dx dy + k2 dy^2 for exp2 and the
+// premultiplied colour; rect = tile rectangle [x0, x1) x [y0, y1); dkey = the bits of its camera depth, which
+// order like z (z > near_z > 0), all ones where it is culled. Returns its tile count (0: culled).
 __device__ __forceinline__ uint32_t splat_one(int64_t i, float px, float py, float pz, const float (&s3)[3], float4 q,
                                               float lg, const float* __restrict__ rgb, const CamDev& cam,
-                                              float4* __restrict__ rec, int4* __restrict__ rect) {
-  uint32_t cnt = 0;
+                                              float4* __restrict__ rec, int4* __restrict__ rect,
+                                              uint32_t* __restrict__ dkey) {
+  uint32_t cnt = 0, key = 0xFFFFFFFFu;
   const float* R = cam.R;
   const float x = fa(dot3(R[0], px, R[1], py, R[2], pz), cam.t[0]);
   const float y = fa(dot3(R[3], px, R[4], py, R[5], pz), cam.t[1]);
@@ -106,13 +108,15 @@ __device__ __forceinline__ uint32_t splat_one(int64_t i, float px, float py, flo
         const float L = 1.4426950408889634f;  // log2(e)
         const float ca = Cc / det, cb = -B / det, cc = A / det;
         const float mu = 1.0f / (1.0f + expf(-lg));  // Eq. sigmoid
-        rec[3 * i] = make_float4(u, v, mu, z);
-        rec[3 * i + 1] = make_float4(-0.5f * L * ca, -L * cb, -0.5f * L * cc, 0.0f);
-        rec[3 * i + 2] = make_float4(rgb[3 * i], rgb[3 * i + 1], rgb[3 * i + 2], 0.0f);
+        rec[3 * i] = make_float4(u, v, -0.5f * L * ca, -L * cb);
+        rec[3 * i + 1] = make_float4(-0.5f * L * cc, -mu, rgb[3 * i], rgb[3 * i + 1]);
+        rec[3 * i + 2] = make_float4(rgb[3 * i + 2], 0.0f, 0.0f, 0.0f);
         rect[i] = make_int4(x0, y0, x1, y1);
+        key = __float_as_uint(z);
       }
     }
   }
+  dkey[i] = key;
   return cnt;
 }
 
@@ -120,10 +124,10 @@ __device__ __forceinline__ uint32_t splat_one(int64_t i, float px, float py, flo
 __global__ void k_splat_setup(int64_t n, const float* __restrict__ pos, const float* __restrict__ scale,
                               const float4* __restrict__ rot, const float* __restrict__ logit,
                               const float* __restrict__ rgb, CamDev cam, float4* __restrict__ rec,
-                              int4* __restrict__ rect, uint32_t* __restrict__ count) {
+                              int4* __restrict__ rect, uint32_t* __restrict__ count, uint32_t* __restrict__ dkey) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const float s3[3] = {scale[3 * i], scale[3 * i + 1], scale[3 * i + 2]};
-    count[i] = splat_one(i, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], s3, rot[i], logit[i], rgb, cam, rec, rect);
+    count[i] = splat_one(i, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], s3, rot[i], logit[i], rgb, cam, rec, rect, dkey);
   }
 }
 
@@ -132,7 +136,7 @@ __global__ void k_splat_setup(int64_t n, const float* __restrict__ pos, const fl
 __global__ void k_splat_setup_coded(const int32_t* __restrict__ glist, int64_t n_list, const int32_t* __restrict__ perm,
                                     int64_t n, GeomStreams G, int64_t chunk_slots, const float* __restrict__ rgb,
                                     CamDev cam, float4* __restrict__ rec, int4* __restrict__ rect,
-                                    uint32_t* __restrict__ count) {
+                                    uint32_t* __restrict__ count, uint32_t* __restrict__ dkey) {
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n_list * 16; v += (int64_t)gridDim.x * blockDim.x) {
     const int32_t g = glist[v >> 4];
     if (g < 0) continue;
@@ -144,7 +148,7 @@ __global__ void k_splat_setup_coded(const int32_t* __restrict__ glist, int64_t n
     float t;
     geom_decode(G, s, chunk_slots, p, sc, q, t);
     const float s3[3] = {sc.x, sc.y, sc.z};
-    count[o] = splat_one(o, p.x, p.y, p.z, s3, q, t, rgb, cam, rec, rect);
+    count[o] = splat_one(o, p.x, p.y, p.z, s3, q, t, rgb, cam, rec, rect, dkey);
   }
 }
 
@@ -211,17 +215,6 @@ __global__ void k_chunk_groups(int64_t nc, const uint32_t* __restrict__ vis, con
   }
 }
 
-// Depth keys of the visible Gaussians (culled ones last), for a stable sort that orders them
-// nearest first with equal depths in index order; camera depth > near_z > 0, so the float bits
-// order like z.
-__global__ void k_depth_keys(int64_t n, const float4* __restrict__ rec, const uint32_t* __restrict__ count,
-                             uint64_t* __restrict__ dkey, uint32_t* __restrict__ dval) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    dkey[i] = count[i] ? (uint64_t)__float_as_uint(rec[3 * i].w) : 0xFFFFFFFFull;
-    dval[i] = (uint32_t)i;
-  }
-}
-
 // tile counts in depth order
 __global__ void k_gather_counts(int64_t n, const uint32_t* __restrict__ dval, const uint32_t* __restrict__ count,
                                 uint32_t* __restrict__ out) {
@@ -230,30 +223,69 @@ __global__ void k_gather_counts(int64_t n, const uint32_t* __restrict__ dval, co
 }
 
 // One tile key per overlapped tile, emitted in depth order: a stable sort by tile then leaves every
-// tile's list nearest first (equal depths in index order).
-__global__ void k_splat_keys(int64_t n, const uint32_t* __restrict__ dval, const int4* __restrict__ rect,
-                             const uint32_t* __restrict__ count_sorted, const uint32_t* __restrict__ offset,
-                             int tiles_x, uint64_t* __restrict__ keys, uint32_t* __restrict__ vals) {
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-    if (count_sorted[r] == 0) continue;
-    const uint32_t i = dval[r];
-    const int4 b = rect[i];
-    uint32_t o = offset[r];
-    for (int ty = b.y; ty < b.w; ty++)
-      for (int tx = b.x; tx < b.z; tx++) {
-        keys[o] = (uint64_t)(ty * tiles_x + tx);
-        vals[o] = i;
-        o++;
+// tile's list nearest first (equal depths in index order). A warp takes 32 Gaussians and writes their keys
+// together, 32 consecutive ones per step (a thread writing its own Gaussian's keys touched a sector per key:
+// 0.40 ms for the 29M keys of a 1080p frame of 3M Gaussians).
+template <class K>
+__global__ void __launch_bounds__(256) k_splat_keys(int64_t n, const uint32_t* __restrict__ dval, const int4* __restrict__ rect,
+                                                    const uint32_t* __restrict__ count_sorted,
+                                                    const uint32_t* __restrict__ offset, int tiles_x,
+                                                    K* __restrict__ keys, uint32_t* __restrict__ vals) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t r0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32; r0 < n; r0 += warps * 32) {
+    const int64_t r = r0 + lane;
+    const uint32_t c = r < n ? count_sorted[r] : 0u;
+    const unsigned any = __ballot_sync(0xFFFFFFFFu, c > 0u);
+    if (any == 0u) continue;
+    const uint32_t i = c ? dval[r] : 0u, o = r < n ? offset[r] : 0xFFFFFFFFu;
+    const int4 b = c ? rect[i] : make_int4(0, 0, 1, 1);
+    const int first = b.y * tiles_x + b.x, wide = b.z - b.x;
+    const int last = 31 - __clz(any);
+    const uint32_t begin = __shfl_sync(0xFFFFFFFFu, o, 0), end = __shfl_sync(0xFFFFFFFFu, o + c, last);
+    for (uint32_t e0 = begin; e0 < end; e0 += 32) {
+      const uint32_t e = e0 + lane;
+      // the last lane whose keys start at or before e (lanes without keys share their successor's start)
+      int j = 0;
+#pragma unroll
+      for (int d = 16; d > 0; d >>= 1) {
+        const uint32_t at = __shfl_sync(0xFFFFFFFFu, o, j + d);
+        if (at <= e) j += d;
       }
+      const uint32_t oj = __shfl_sync(0xFFFFFFFFu, o, j), ij = __shfl_sync(0xFFFFFFFFu, i, j);
+      const int fj = __shfl_sync(0xFFFFFFFFu, first, j), wj = __shfl_sync(0xFFFFFFFFu, wide, j);
+      if (e < end) {
+        const int k = (int)(e - oj), row = k / wj;
+        keys[e] = (K)(fj + row * tiles_x + (k - row * wj));
+        vals[e] = ij;
+      }
+    }
   }
 }
 
-// ranges[tile] = [first, last + 1) of the tile's entries in the sorted list (empty tiles stay 0)
-__global__ void k_tile_ranges(const uint64_t* __restrict__ keys, int64_t P, uint2* __restrict__ ranges) {
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < P; e += (int64_t)gridDim.x * blockDim.x) {
-    const uint32_t t = (uint32_t)keys[e];
-    if (e == 0 || (uint32_t)keys[e - 1] != t) ranges[t].x = (uint32_t)e;
-    if (e == P - 1 || (uint32_t)keys[e + 1] != t) ranges[t].y = (uint32_t)(e + 1);
+// ranges[tile] = [first, last + 1) of the tile's entries in the sorted list (empty tiles stay 0). Every key is read
+// once, its neighbours' come by shuffle.
+template <class K>
+__global__ void __launch_bounds__(256) k_tile_ranges(const K* __restrict__ keys, int64_t P, uint2* __restrict__ ranges) {
+  const int lane = threadIdx.x & 31;
+  const int64_t step = (int64_t)gridDim.x * (blockDim.x >> 5) * 128;
+  for (int64_t b = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 128; b < P; b += step) {
+    uint32_t t[4], before[4], after[4];
+#pragma unroll
+    for (int q = 0; q < 4; q++) t[q] = b + 32 * q + lane < P ? (uint32_t)keys[b + 32 * q + lane] : 0xFFFFFFFFu;
+    const uint32_t left = b > 0 ? (uint32_t)keys[b - 1] : 0xFFFFFFFFu, right = b + 128 < P ? (uint32_t)keys[b + 128] : 0xFFFFFFFFu;
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      before[q] = __shfl_up_sync(0xFFFFFFFFu, t[q], 1);
+      after[q] = __shfl_down_sync(0xFFFFFFFFu, t[q], 1);
+      const uint32_t l = q > 0 ? __shfl_sync(0xFFFFFFFFu, t[q > 0 ? q - 1 : 0], 31) : left;
+      const uint32_t r = q < 3 ? __shfl_sync(0xFFFFFFFFu, t[q < 3 ? q + 1 : 3], 0) : right;
+      if (lane == 0) before[q] = l;
+      if (lane == 31) after[q] = r;
+      const int64_t e = b + 32 * q + lane;
+      if (e < P && before[q] != t[q]) ranges[t[q]].x = (uint32_t)e;
+      if (e < P && after[q] != t[q]) ranges[t[q]].y = (uint32_t)(e + 1);
+    }
   }
 }
 
@@ -265,64 +297,149 @@ __device__ __forceinline__ float ex2(float x) {
   return r;
 }
 
-// Eq. preblend per pixel, the tile's Gaussians nearest first, staged 256 at a time in shared
-// memory; 128 threads, each blending two pixels of one tile column (rows y and y + 8) with one
-// read of every staged splat (four pixels per thread on 64 threads measured slower: 5.05 against
-// 4.33 ms at 1080p). With w = T g, the transmittance update T (1 - mu g) is T - mu w.
-#define RTHREADS 128
-#define RPIX 2
-#define RSTEP 8
-#define RBATCH 256
-__global__ void __launch_bounds__(RTHREADS) k_render(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals,
-                                                     const float4* __restrict__ rec, int width, int height, int tiles_x,
-                                                     float* __restrict__ image, float* __restrict__ trans) {
-  __shared__ float4 s0[RBATCH], s1[RBATCH], s2[RBATCH];
-  const int tile = blockIdx.x;
+// Eq. preblend per pixel, the tile's Gaussians nearest first. With w = T g, the transmittance update
+// T (1 - mu g) is T - mu w. A warp owns a tile: lane l the eight pixels of column l % 16 whose rows have the
+// parity l / 16, in four pairs for the two-lane multiply-adds. The exponent at row y0 + c is
+// q(y0) + c (2 k2 dy0 + k1 dx) + c^2 k2, two multiply-adds per pixel pair. Records are staged 32 at a time
+// through shared memory, the next 32 loaded while these are blended. Bound by the multiply-add pipe (70% busy; a
+// splat is 28 two-lane instructions of two cycles and 10 others per warp): 2.2 ms for the 29M (Gaussian, tile)
+// pairs of a 1080p frame of 3M Gaussians, against 4.5 ms with four warps per tile and two pixels per thread,
+// which issued 15 instructions per pixel and read every splat four times.
+//
+// Blending is associative: a run of splats takes (colour, T) to (colour + T C', T T') with the run's own C' and
+// T'. Lists longer than RSEG are cut into segments of RSEG, each a warp's job with its result in a slot, joined
+// in order by k_render_join: a 1080p frame of 3M clustered Gaussians has lists of 3,500 on average and of tens
+// of thousands in the middle, and one warp per list left the machine waiting for the longest (5.3 ms).
+#define RROWS 8
+#define RSTAGE 32
+#define RSEG 1024
+struct Segment { uint32_t tile, seg; };
+struct Split { uint32_t tile, first, count; };  // a long list's slots
+
+// Segments of the lists longer than RSEG. n_out[0]: segments, n_out[1]: such lists.
+__global__ void k_render_split(const uint2* __restrict__ ranges, int64_t tiles, Segment* __restrict__ segs,
+                               Split* __restrict__ splits, uint32_t* __restrict__ n_out) {
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < tiles; t += (int64_t)gridDim.x * blockDim.x) {
+    const uint2 rg = ranges[t];
+    const uint32_t len = rg.y - rg.x;
+    if (len <= RSEG) continue;
+    const uint32_t c = (len + RSEG - 1) / RSEG, x = atomicAdd(&n_out[0], c);
+    splits[atomicAdd(&n_out[1], 1u)] = {(uint32_t)t, x, c};
+    for (uint32_t i = 0; i < c; i++) segs[x + i] = {(uint32_t)t, i};
+  }
+}
+
+// One CTA per long list: its segments joined, nearest first.
+__global__ void __launch_bounds__(256) k_render_join(const Split* __restrict__ splits, const uint32_t* __restrict__ n_split,
+                                                    const float4* __restrict__ slots, int width, int height, int tiles_x,
+                                                    float* __restrict__ image, float* __restrict__ trans) {
+  if (blockIdx.x >= *n_split) return;
+  const Split s = splits[blockIdx.x];
+  const int px = (int)(s.tile % tiles_x) * RTILE + (threadIdx.x & 15), py = (int)(s.tile / tiles_x) * RTILE + (threadIdx.x >> 4);
+  float4 c = make_float4(0.f, 0.f, 0.f, 1.f);
+  for (uint32_t i = 0; i < s.count; i++) {
+    const float4 v = slots[(int64_t)(s.first + i) * 256 + threadIdx.x];
+    c.x += c.w * v.x; c.y += c.w * v.y; c.z += c.w * v.z;
+    c.w *= v.w;
+  }
+  if (px < width && py < height) {
+    const int64_t p = (int64_t)py * width + px;
+    image[3 * p] = c.x;
+    image[3 * p + 1] = c.y;
+    image[3 * p + 2] = c.z;
+    if (trans) trans[p] = c.w;
+  }
+}
+
+// CTAs [0, tiles): the lists of up to RSEG; CTAs from tiles on: the segments.
+__global__ void __launch_bounds__(32) k_render(const uint2* __restrict__ ranges, const uint32_t* __restrict__ vals,
+                                               const float4* __restrict__ rec, const Segment* __restrict__ segs,
+                                               const uint32_t* __restrict__ n_segs, int tiles, int width, int height,
+                                               int tiles_x, float4* __restrict__ slots, float* __restrict__ image,
+                                               float* __restrict__ trans) {
+  // (u, v, k0, k1); then each value twice, as the two-lane multiply-adds take them: (k2, -mu), (r, g), b
+  __shared__ float4 s0[RSTAGE], s1[RSTAGE], s2[RSTAGE];
+  __shared__ float2 s3[RSTAGE];
+  const int lane = threadIdx.x;
+  int tile = blockIdx.x, slot = -1;
+  uint2 rg;
+  if (tile < tiles) {
+    rg = ranges[tile];
+    if (rg.y - rg.x > RSEG) return;
+  } else {
+    slot = tile - tiles;
+    if (slot >= (int)*n_segs) return;
+    const Segment s = segs[slot];
+    tile = (int)s.tile;
+    rg = ranges[tile];
+    rg.x += s.seg * RSEG;
+    rg.y = min(rg.y, rg.x + RSEG);
+  }
   const int tx = tile % tiles_x, ty = tile / tiles_x;
-  const int px = tx * RTILE + (threadIdx.x & (RTILE - 1)), py = ty * RTILE + (threadIdx.x / RTILE);
+  const int px = tx * RTILE + (lane & 15), py = ty * RTILE + (lane >> 4);  // rows py, py + 2, .. py + 14
   const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
-  const uint2 rg = ranges[tile];
-  float T[RPIX], r[RPIX], g[RPIX], b[RPIX];
+  float2 T[RROWS / 2], r[RROWS / 2], g[RROWS / 2], b[RROWS / 2];
 #pragma unroll
-  for (int j = 0; j < RPIX; j++) { T[j] = 1.0f; r[j] = 0.0f; g[j] = 0.0f; b[j] = 0.0f; }
-  for (uint32_t e0 = rg.x; e0 < rg.y; e0 += RBATCH) {
-    __syncthreads();
-#pragma unroll
-    for (int h = 0; h < RBATCH / RTHREADS; h++) {
-      const uint32_t e = e0 + h * RTHREADS + threadIdx.x;
-      if (e < rg.y) {
-        const uint32_t i = vals[e];
-        s0[h * RTHREADS + threadIdx.x] = rec[3 * (int64_t)i];
-        s1[h * RTHREADS + threadIdx.x] = rec[3 * (int64_t)i + 1];
-        s2[h * RTHREADS + threadIdx.x] = rec[3 * (int64_t)i + 2];
-      }
-    }
-    __syncthreads();
-    const int m = (int)min((uint32_t)RBATCH, rg.y - e0);
+  for (int j = 0; j < RROWS / 2; j++) {
+    T[j] = make_float2(1.0f, 1.0f);
+    r[j] = g[j] = b[j] = make_float2(0.0f, 0.0f);
+  }
+  // entry indices two stages ahead, records one
+  uint32_t id = rg.x + lane < rg.y ? vals[rg.x + lane] : 0u;
+  float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
+  float n2 = 0.f;
+  if (rg.x + lane < rg.y) { const float4* p = rec + 3 * (int64_t)id; n0 = p[0]; n1 = p[1]; n2 = p[2].x; }
+  id = rg.x + RSTAGE + lane < rg.y ? vals[rg.x + RSTAGE + lane] : 0u;
+  for (uint32_t e0 = rg.x; e0 < rg.y; e0 += RSTAGE) {
+    __syncwarp();
+    s0[lane] = n0;
+    s1[lane] = make_float4(n1.x, n1.x, n1.y, n1.y);
+    s2[lane] = make_float4(n1.z, n1.z, n1.w, n1.w);
+    s3[lane] = make_float2(n2, n2);
+    __syncwarp();
+    if (e0 + RSTAGE + lane < rg.y) { const float4* p = rec + 3 * (int64_t)id; n0 = p[0]; n1 = p[1]; n2 = p[2].x; }
+    if (e0 + 2 * RSTAGE + lane < rg.y) id = vals[e0 + 2 * RSTAGE + lane];
+    const int m = (int)min((uint32_t)RSTAGE, rg.y - e0);
+#pragma unroll 8
     for (int k = 0; k < m; k++) {
-      const float4 a = s0[k], c = s1[k], col = s2[k];
+      const float4 a = s0[k], c = s1[k], d = s2[k];
+      const float2 k2 = make_float2(c.x, c.y), nm = make_float2(c.z, c.w);
+      const float2 cr = make_float2(d.x, d.y), cg = make_float2(d.z, d.w), cb = s3[k];
       const float dx = fx - a.x, dy = fy - a.y;
-      const float qx = c.x * dx;  // the exponent is dx (k0 dx + k1 dy) + k2 dy^2
+      const float k1dx = a.w * dx, sum = fmaf(c.x, dy, k1dx), slope = fmaf(c.x, dy, sum);
+      const float q0 = fmaf(dy, sum, dx * (a.z * dx));
+      const float2 q2 = make_float2(q0, q0), sl = make_float2(slope, slope);
 #pragma unroll
-      for (int j = 0; j < RPIX; j++) {
-        const float d = dy + (float)(RSTEP * j);
-        const float q = dx * (qx + c.y * d) + c.z * d * d;
-        const float w = T[j] * ex2(q);
-        r[j] += w * col.x;
-        g[j] += w * col.y;
-        b[j] += w * col.z;
-        T[j] -= a.z * w;
+      for (int j = 0; j < RROWS / 2; j++) {
+        const float y0 = (float)(4 * j), y1 = (float)(4 * j + 2);  // row offsets of the pair
+        const float2 q = __ffma2_rn(make_float2(y0, y1), sl, __ffma2_rn(make_float2(y0 * y0, y1 * y1), k2, q2));
+        const float2 w = __fmul2_rn(T[j], make_float2(ex2(q.x), ex2(q.y)));
+        r[j] = __ffma2_rn(w, cr, r[j]);
+        g[j] = __ffma2_rn(w, cg, g[j]);
+        b[j] = __ffma2_rn(w, cb, b[j]);
+        T[j] = __ffma2_rn(w, nm, T[j]);
       }
     }
   }
+  if (slot >= 0) {
 #pragma unroll
-  for (int j = 0; j < RPIX; j++) {
-    if (px < width && py + RSTEP * j < height) {
-      const int64_t p = (int64_t)(py + RSTEP * j) * width + px;
-      image[3 * p] = r[j];
-      image[3 * p + 1] = g[j];
-      image[3 * p + 2] = b[j];
-      if (trans) trans[p] = T[j];
+    for (int j = 0; j < RROWS; j++) {
+      const int h = j >> 1;
+      slots[(int64_t)slot * 256 + ((lane >> 4) + 2 * j) * RTILE + (lane & 15)] =
+          j & 1 ? make_float4(r[h].y, g[h].y, b[h].y, T[h].y) : make_float4(r[h].x, g[h].x, b[h].x, T[h].x);
+    }
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < RROWS; j++) {
+    const int y = py + 2 * j;
+    if (px < width && y < height) {
+      const int64_t p = (int64_t)y * width + px;
+      const int h = j >> 1;
+      image[3 * p] = j & 1 ? r[h].y : r[h].x;
+      image[3 * p + 1] = j & 1 ? g[h].y : g[h].x;
+      image[3 * p + 2] = j & 1 ? b[h].y : b[h].x;
+      if (trans) trans[p] = j & 1 ? T[h].y : T[h].x;
     }
   }
 }
@@ -357,14 +474,14 @@ struct RenderWs {
   uint64_t* total;
   void* scan_ws;
   uint2* ranges;
-  uint64_t* dkey;
+  uint32_t *dkey, *dkey2;  // depth keys and the sort's second array
   uint32_t *dval, *count_sorted;
   uint32_t *vis, *vrank;
   int32_t* glist;
   float* pos_dec;
-  uint64_t* keys;
-  uint32_t* vals;
-  void* radix_ws;
+  uint32_t *keys, *keys2;  // tile keys and the sort's second array
+  uint32_t *vals, *vals2;  // vals2: of either sort
+  void* radix_state;
 };
 
 // fixed part first, then the buffers that grow with the number of (Gaussian, tile) pairs
@@ -381,16 +498,20 @@ RenderWs carve_render(void* ws, size_t cap, int64_t n, int64_t tiles, int64_t pa
   w.total = c.take<uint64_t>(1);
   w.scan_ws = c.take<uint8_t>((int64_t)scan_ws_bytes(n));
   w.ranges = c.take<uint2>(tiles);
-  w.dkey = c.take<uint64_t>(n);
+  w.dkey = c.take<uint32_t>(2 * n);
+  w.dkey2 = w.dkey + n;
   w.dval = c.take<uint32_t>(n);
   w.count_sorted = c.take<uint32_t>(n);
   w.vis = c.take<uint32_t>(nc);
   w.vrank = c.take<uint32_t>(nc);
   w.glist = c.take<int32_t>(ng);
   w.pos_dec = c.take<float>(ng > 0 ? 3 * n : 0);
-  w.keys = c.take<uint64_t>(pairs);
+  w.keys = c.take<uint32_t>(2 * pairs);
+  w.keys2 = w.keys + pairs;
   w.vals = c.take<uint32_t>(pairs);
-  w.radix_ws = c.take<uint8_t>((int64_t)radix_ws_bytes(pairs > n ? pairs : n));
+  const int64_t most = pairs > n ? pairs : n;
+  w.vals2 = c.take<uint32_t>(most);
+  w.radix_state = c.take<uint8_t>((int64_t)radix_state_bytes(most));
   *ok = c.ok();
   return w;
 }
@@ -416,7 +537,8 @@ size_t render_bytes(int64_t n, int64_t tiles, int64_t pairs, int64_t nc, int64_t
   add(ng > 0 ? 12 * n : 0);
   add(8 * pairs);
   add(4 * pairs);
-  add((int64_t)radix_ws_bytes(pairs > n ? pairs : n));
+  add(4 * (pairs > n ? pairs : n));
+  add((int64_t)radix_state_bytes(pairs > n ? pairs : n));
   return align_up(b, 256) + 256;
 }
 
@@ -431,6 +553,22 @@ extern "C" size_t gsc_render_workspace_bytes(int64_t n, const gsc_camera* cam, i
 }
 
 namespace {
+
+// every tile's list, nearest first: keys emitted in depth order, sorted by tile; *lists: where the sorted values are
+template <class K>
+cudaError_t tile_lists(const RenderWs& w, int64_t n, int64_t pairs, int tiles_x, int64_t tiles, cudaStream_t st,
+                       uint32_t** lists) {
+  K *keys = reinterpret_cast<K*>(w.keys), *keys2 = reinterpret_cast<K*>(w.keys2), *sorted;
+  gsc_count_launch();
+  k_splat_keys<K><<<grid_of(n), 256, 0, st>>>(n, w.dval, w.rect, w.count_sorted, w.offset, tiles_x, keys, w.vals);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess)
+    e = radix_sort<K>(keys, keys2, w.vals, w.vals2, pairs, tile_bits(tiles), false, true, w.radix_state, st, &sorted, lists);
+  if (e != cudaSuccess) return e;
+  gsc_count_launch();
+  k_tile_ranges<K><<<grid_of(pairs), 256, 0, st>>>(sorted, pairs, w.ranges);
+  return cudaGetLastError();
+}
 
 // The shared pipeline: colour (fused decode + SH for the camera centre), splat setup (float geometry,
 // or the streams of the kept chunks), depth sort, tile keys, tile sort, ranges, blending.
@@ -482,6 +620,7 @@ gsc_status render_run(gsc_ctx* c, const DevTable& T, const uint8_t* d_blocks, co
       kept = *hcount;
       const int64_t n_list = (int64_t)kept * gpc - (*hlast ? nc * gpc - ng : 0);
       GSC_CUDA(cudaMemsetAsync(w.count, 0, sizeof(uint32_t) * (size_t)n, st));
+      GSC_CUDA(cudaMemsetAsync(w.dkey, 0xFF, sizeof(uint32_t) * (size_t)n, st));
       if (n_list > 0) {
         gsc_count_launch();
         k_decode_positions<<<grid_of(n_list * 16), 256, 0, st>>>(w.glist, n_list, d_perm, n, G, chunk_slots,
@@ -491,21 +630,19 @@ gsc_status render_run(gsc_ctx* c, const DevTable& T, const uint8_t* d_blocks, co
                                     c->sm_count, st, w.glist, n_list));
         gsc_count_launch();
         k_splat_setup_coded<<<grid_of(n_list * 16), 256, 0, st>>>(w.glist, n_list, d_perm, n, G, chunk_slots, w.rgb,
-                                                                   cd, w.rec, w.rect, w.count);
+                                                                   cd, w.rec, w.rect, w.count, w.dkey);
         GSC_CUDA(cudaGetLastError());
       }
     } else {
       GSC_CUDA(launch_decode_eval(T, d_blocks, d_perm, nullptr, d_pos, w.f, 1, GSC_OUT_GAUSS_MAJOR, w.rgb, c->sm_count, st));
       gsc_count_launch();
       k_splat_setup<<<grid_of(n), 256, 0, st>>>(n, d_pos, d_scale, reinterpret_cast<const float4*>(d_rot), d_logit,
-                                               w.rgb, cd, w.rec, w.rect, w.count);
+                                               w.rgb, cd, w.rec, w.rect, w.count, w.dkey);
       GSC_CUDA(cudaGetLastError());
     }
     // visible Gaussians nearest first (stable: equal depths in index order), their counts in that order
-    gsc_count_launch();
-    k_depth_keys<<<grid_of(n), 256, 0, st>>>(n, w.rec, w.count, w.dkey, w.dval);
-    GSC_CUDA(cudaGetLastError());
-    GSC_CUDA(radix_sort_pairs(w.dkey, w.dval, n, 32, w.radix_ws, st));
+    uint32_t *dk, *dv;  // four passes: the result is back in dval, which the pair buffers do not touch
+    GSC_CUDA(radix_sort<uint32_t>(w.dkey, w.dkey2, w.dval, w.vals2, n, 32, true, false, w.radix_state, st, &dk, &dv));
     gsc_count_launch();
     k_gather_counts<<<grid_of(n), 256, 0, st>>>(n, w.dval, w.count, w.count_sorted);
     GSC_CUDA(cudaGetLastError());
@@ -519,21 +656,35 @@ gsc_status render_run(gsc_ctx* c, const DevTable& T, const uint8_t* d_blocks, co
   if (pairs > 0xFFFFFFF0ull) return GSC_ERR_OOM;
   w = carve_render(d_ws, ws_bytes, n, tiles, (int64_t)pairs, coded ? ng : 0, coded ? ng : 0, &ok);
   if (!ok) return GSC_ERR_OOM;
+  uint32_t* lists = w.vals;
   if (pairs > 0) {
-    gsc_count_launch();
-    k_splat_keys<<<grid_of(n), 256, 0, st>>>(n, w.dval, w.rect, w.count_sorted, w.offset, cd.tiles_x, w.keys,
-                                             w.vals);
-    GSC_CUDA(cudaGetLastError());
-    GSC_CUDA(radix_sort_pairs(w.keys, w.vals, (int64_t)pairs, tile_bits(tiles), w.radix_ws, st));
-    gsc_count_launch();
-    k_tile_ranges<<<grid_of((int64_t)pairs), 256, 0, st>>>(w.keys, (int64_t)pairs, w.ranges);
-    GSC_CUDA(cudaGetLastError());
+    // 16-bit tile keys where the image has that few tiles: a third less to move per pass of the sort
+    if (tiles <= 65536) GSC_CUDA((tile_lists<uint16_t>(w, n, (int64_t)pairs, cd.tiles_x, tiles, st, &lists)));
+    else GSC_CUDA((tile_lists<uint32_t>(w, n, (int64_t)pairs, cd.tiles_x, tiles, st, &lists)));
   }
   GscTimed tb(c, T_BLEND, st);
+  // a long list has more than RSEG entries: at most pairs / RSEG of them, and twice that many segments. The slots (4 KB
+  // each) take the tile keys' two arrays, the tables the values' array that the sort left over.
+  const int64_t most = (int64_t)pairs / RSEG;
+  float4* slots = reinterpret_cast<float4*>(w.keys);
+  Segment* segs = reinterpret_cast<Segment*>(lists == w.vals ? w.vals2 : w.vals);
+  Split* splits = reinterpret_cast<Split*>(segs + 2 * most);
+  uint32_t* n_out = reinterpret_cast<uint32_t*>(w.total);
+  if (most > 0) {
+    GSC_CUDA(cudaMemsetAsync(n_out, 0, 2 * sizeof(uint32_t), st));
+    gsc_count_launch();
+    k_render_split<<<grid_of(tiles), 256, 0, st>>>(w.ranges, tiles, segs, splits, n_out);
+    GSC_CUDA(cudaGetLastError());
+  }
   gsc_count_launch();
-  k_render<<<(int)tiles, RTHREADS, 0, st>>>(w.ranges, w.vals, w.rec, cam->width, cam->height, cd.tiles_x, d_image,
-                                           d_trans);
+  k_render<<<(int)(tiles + 2 * most), 32, 0, st>>>(w.ranges, lists, w.rec, segs, n_out, (int)tiles, cam->width,
+                                                  cam->height, cd.tiles_x, slots, d_image, d_trans);
   GSC_CUDA(cudaGetLastError());
+  if (most > 0) {
+    gsc_count_launch();
+    k_render_join<<<(int)most, 256, 0, st>>>(splits, n_out + 1, slots, cam->width, cam->height, cd.tiles_x, d_image, d_trans);
+    GSC_CUDA(cudaGetLastError());
+  }
   return GSC_OK;
 }
 

@@ -175,15 +175,17 @@ __global__ void __launch_bounds__(256) k_rs_rows(uint32_t* __restrict__ counts, 
 }
 
 // vin = nullptr: values are the input positions; kout = nullptr: the sorted keys are not wanted
-template <class K>
-__global__ void __launch_bounds__(RS_THREADS, sizeof(K) == 4 ? 4 : 3)
-    k_rs_scatter(const K* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t n, int shift, uint32_t mask,
+template <class K, int BITS>
+__global__ void __launch_bounds__(RS_THREADS, sizeof(K) <= 4 ? 4 : 3)
+    k_rs_scatter(const K* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t n, int shift,
                  const uint32_t* __restrict__ total, const uint32_t* __restrict__ counts, K* __restrict__ kout,
                  uint32_t* __restrict__ vout) {
-  __shared__ K s_item[RS_TILE];  // the sorted keys, then the sorted values
+  __shared__ uint64_t s_items[RS_TILE * (sizeof(K) > 4 ? sizeof(K) : 4) / 8];
+  K* s_item = reinterpret_cast<K*>(s_items);  // the sorted keys, then the sorted values
   __shared__ uint32_t s_cnt[RS_WARPS][256];
   __shared__ uint32_t s_start[256], s_base[256];
   __shared__ uint64_t s_scan[8];
+  constexpr uint32_t mask = (1u << BITS) - 1u;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int64_t base = (int64_t)blockIdx.x * RS_TILE;
   const int count = (int)min((int64_t)RS_TILE, n - base);
@@ -194,7 +196,7 @@ __global__ void __launch_bounds__(RS_THREADS, sizeof(K) == 4 ? 4 : 3)
 #pragma unroll
   for (int r = 0; r < RS_ITEMS; r++) key[r] = first + 32 * r < count ? kin[base + first + 32 * r] : (K)0;
   auto digit = [&](int r) { return first + 32 * r < count ? (uint32_t)(key[r] >> shift) & mask : 256u; };
-  const uint32_t mine = rank_digits<RS_WARPS, RS_ITEMS>(digit, rank, s_cnt);
+  const uint32_t mine = rank_digits<RS_WARPS, RS_ITEMS, BITS>(digit, rank, s_cnt);
   // where digit t starts in the output and in the tile
   const uint64_t both = prefix256(((uint64_t)all << 16) | mine, s_scan);
   const uint32_t start = (uint32_t)(both & 0xFFFFu);
@@ -238,14 +240,19 @@ cudaError_t radix_sort(K* keys, K* keys2, uint32_t* vals, uint32_t* vals2, int64
   uint32_t* total = reinterpret_cast<uint32_t*>(state);
   uint32_t* counts = total + 256;
   const int nt = (int)rs_tiles(n);
-  for (int p = 0; p < passes && n > 0; p++) {
-    const int left = key_bits - 8 * p;
-    const uint32_t mask = left >= 8 ? 255u : (1u << left) - 1u;
-    gsc_count_launch(); k_rs_count<K><<<nt, RS_THREADS, 0, st>>>(keys, n, 8 * p, mask, counts);
+  // the key's bits in equal shares of at most 8
+  for (int p = 0, shift = 0; p < passes && n > 0; p++) {
+    const int bits = (key_bits - shift + passes - p - 1) / (passes - p);
+    gsc_count_launch(); k_rs_count<K><<<nt, RS_THREADS, 0, st>>>(keys, n, shift, (1u << bits) - 1u, counts);
     gsc_count_launch(); k_rs_rows<<<256, 256, 0, st>>>(counts, nt, total);
     gsc_count_launch();
-    k_rs_scatter<K><<<nt, RS_THREADS, 0, st>>>(keys, p == 0 && iota ? nullptr : vals, n, 8 * p, mask, total, counts,
-                                               p + 1 < passes || want_keys ? keys2 : nullptr, vals2);
+    const uint32_t* vin = p == 0 && iota ? nullptr : vals;
+    K* kout = p + 1 < passes || want_keys ? keys2 : nullptr;
+    if (bits <= 4) k_rs_scatter<K, 4><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, shift, total, counts, kout, vals2);
+    else if (bits <= 6) k_rs_scatter<K, 6><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, shift, total, counts, kout, vals2);
+    else if (bits == 7) k_rs_scatter<K, 7><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, shift, total, counts, kout, vals2);
+    else k_rs_scatter<K, 8><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, shift, total, counts, kout, vals2);
+    shift += bits;
     K* tk = keys; keys = keys2; keys2 = tk;
     uint32_t* tv = vals; vals = vals2; vals2 = tv;
   }
@@ -253,6 +260,8 @@ cudaError_t radix_sort(K* keys, K* keys2, uint32_t* vals, uint32_t* vals2, int64
   *out_vals = vals;
   return cudaGetLastError();
 }
+template cudaError_t radix_sort<uint16_t>(uint16_t*, uint16_t*, uint32_t*, uint32_t*, int64_t, int, bool, bool, void*, cudaStream_t,
+                                          uint16_t**, uint32_t**);
 template cudaError_t radix_sort<uint32_t>(uint32_t*, uint32_t*, uint32_t*, uint32_t*, int64_t, int, bool, bool, void*, cudaStream_t,
                                           uint32_t**, uint32_t**);
 template cudaError_t radix_sort<uint64_t>(uint64_t*, uint64_t*, uint32_t*, uint32_t*, int64_t, int, bool, bool, void*, cudaStream_t,

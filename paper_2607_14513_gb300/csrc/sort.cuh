@@ -22,13 +22,13 @@ __device__ __forceinline__ uint64_t prefix256(uint64_t v, uint64_t* s) {
   return before;
 }
 
-// Stable ranks of a CTA's items by an 8-bit digit. Warp w holds ITEMS * 32 consecutive items, item r of lane l
+// Stable ranks of a CTA's items by a digit of BITS (at most 8) bits. Warp w holds ITEMS * 32 consecutive items, item r of lane l
 // being r * 32 + l of them; digit(r) = 256 for an item past the end. On return rank[r] is the item's position
 // among its warp's items of the same digit, and cnt[w][d] the number of items of digit d in the warps before w;
-// the total per digit is returned to thread d < 256. cnt has WARPS rows. A round's peers come from eight ballots
+// the total per digit is returned to thread d < 256. cnt has WARPS rows. A round's peers come from BITS ballots
 // (a match instruction took several times as long on digits that mostly differ), and its leaders take their
 // places with one shared-memory addition each: rounds wait neither for one another nor for a barrier.
-template <int WARPS, int ITEMS, class Digit>
+template <int WARPS, int ITEMS, int BITS, class Digit>
 __device__ __forceinline__ uint32_t rank_digits(Digit digit, uint32_t (&rank)[ITEMS], uint32_t (*cnt)[256]) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t below = (1u << lane) - 1u;
@@ -41,7 +41,7 @@ __device__ __forceinline__ uint32_t rank_digits(Digit digit, uint32_t (&rank)[IT
     const bool live = d < 256u;
     uint32_t peers = __ballot_sync(0xFFFFFFFFu, live);
 #pragma unroll
-    for (int b = 0; b < 8; b++) {
+    for (int b = 0; b < BITS; b++) {
       const uint32_t set = __ballot_sync(0xFFFFFFFFu, (d >> b) & 1u);
       peers &= (d >> b) & 1u ? set : ~set;
     }
