@@ -192,10 +192,10 @@ __global__ void __launch_bounds__(32 * BC7_WARPS, BC7_MIN_BLOCKS)
           int64_t n_groups, const uint8_t* __restrict__ texin, int64_t nblk, uint4* __restrict__ blocks,
           uint32_t* __restrict__ sse7, uint64_t* __restrict__ sse64) {
   __shared__ Bc7Warp S[BC7_WARPS];
-  __shared__ float s_scale[16];
+  __shared__ StageScale T;
   __shared__ uint8_t sq[12 * 256];
   for (int i = threadIdx.x; i < 12 * 256; i += blockDim.x) sq[i] = (&g_qtab[0][0])[i];
-  if (!texin && threadIdx.x < 16) s_scale[threadIdx.x] = scales[threadIdx.x];
+  if (!texin && threadIdx.x < 32) stage_scales(T, scales);
   __syncthreads();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t total = texin ? nblk : n_groups * 16;
@@ -206,7 +206,8 @@ __global__ void __launch_bounds__(32 * BC7_WARPS, BC7_MIN_BLOCKS)
     if (!texin) {
       // two groups, or the one that holds the warp's eight blocks
       const int64_t g0 = b0 / 16;
-      stage_groups<BC7_STRIDE, 1>(sh, perm, s_scale, g0, BPW == 32 ? n_groups : g0 + 1, S[w].tex, lane);
+      stage_groups<BC7_STRIDE, 1>(sh, perm, T, g0, BPW == 32 ? n_groups : g0 + 1, S[w].tex,
+                                  reinterpret_cast<uint32_t*>(S[w].r));
       col0 = (int)(b0 - g0 * 16);
     } else if (live) {
       const uint8_t* p = texin + blk * 48;
@@ -251,12 +252,19 @@ cudaError_t launch_bc7_blocks(const uint8_t* tex, int64_t nblk, uint8_t* out, ui
 }
 
 // ---- persistent multi-scene encode -----------------------------------------------------------
-// One launch per coding (KIND 1 = BC1, 7 = BC7) over the tiles of every listed scene. Tiles
+// One launch per coding over the tiles of every listed scene. Tiles
 // are claimed round robin (schedule 0), from an atomic work queue (1, 2), or one per claiming unit
-// (3, a grid of all tiles); a tile finds its scene by binary search over the list. A BC1 CTA of 128
-// threads claims as a whole; the four warps of a BC7 CTA claim their own tiles and walk them two
-// groups (32 blocks) at a time, since their searches differ in length. The bits equal the
-// single-scene kernels'.
+// (3, a grid of all tiles); a tile finds its scene by binary search over the list. The four warps of a CTA claim
+// their own tiles and walk them 8 groups (BC1) or two (BC7) at a time, since their searches differ in length. The
+// bits equal the single-scene kernels'.
+__device__ __forceinline__ int64_t claim_tile(int schedule, int64_t it, int w, int lane, int* counter) {
+  long long ti = 0;
+  if (lane == 0)
+    ti = (schedule == 0 || schedule == 3) ? (long long)((blockIdx.x + it * gridDim.x) * BC7_WARPS + w)
+                                          : (long long)atomicAdd(counter, 1);
+  return __shfl_sync(0xFFFFFFFFu, ti, 0);
+}
+
 __device__ __forceinline__ BatchSceneDev scene_of(const BatchSceneDev* __restrict__ scenes, int n_scenes, int64_t ti) {
   int lo = 0, hi = n_scenes - 1;
   while (lo < hi) {
@@ -266,38 +274,26 @@ __device__ __forceinline__ BatchSceneDev scene_of(const BatchSceneDev* __restric
   return scenes[lo];
 }
 
-__global__ void __launch_bounds__(STAGE_THREADS, BC7_MIN_BLOCKS)
+__global__ void __launch_bounds__(32 * BC7_WARPS, 4)
     k_batch1(const BatchSceneDev* __restrict__ scenes, int n_scenes, int64_t n_tiles, int schedule,
              int* __restrict__ counter) {
-  __shared__ uint32_t tex[16][STAGE_STRIDE];
-  __shared__ float s_scale[16];
-  __shared__ long long s_tile;
-  const int lt = threadIdx.x;
+  __shared__ Bc1Warp<128> W[BC7_WARPS];
+  __shared__ StageScale T[BC7_WARPS];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int64_t it = 0;; it++) {
-    __syncthreads();
-    if (lt == 0)
-      s_tile = (schedule == 0 || schedule == 3) ? (long long)(blockIdx.x + it * gridDim.x) : (long long)atomicAdd(counter, 1);
-    __syncthreads();
-    const int64_t ti = s_tile;
+    const int64_t ti = claim_tile(schedule, it, w, lane, counter);
     if (ti >= n_tiles) break;
     const BatchSceneDev S = scene_of(scenes, n_scenes, ti);
     const int64_t gbeg = (ti - S.tile0) * S.tile_groups, gend = min(gbeg + (int64_t)S.tile_groups, S.work_groups);
-    if (lt < 16) s_scale[lt] = S.scales[lt];
-    __syncthreads();
-    for (int64_t g0 = gbeg; g0 < gend; g0 += STAGE_GROUPS) {
-      stage_groups<STAGE_STRIDE>(S.sh, S.perm, s_scale, g0, S.n_groups, tex, lt);
-      __syncthreads();
-      const int64_t blk = g0 * 16 + lt;
-      if (blk < S.n_groups * 16) {
-        uint32_t tx[16];
-#pragma unroll
-        for (int t = 0; t < 16; t++) tx[t] = tex[t][lt];
-        const Bc1Res r = bc1_encode(tx);
-        reinterpret_cast<uint2*>(S.b1)[blk] = bc1_bits(r);
-        if (S.sse1) S.sse1[blk] = r.sse;
-        if (S.sse0) S.sse0[blk] = sse_zero(tx);
-      }
-      __syncthreads();
+    stage_scales(T[w], S.scales);
+    __syncwarp();
+    for (int64_t g0 = gbeg; g0 < gend; g0 += 8) {
+#pragma unroll 1
+      for (int i = 0; i < 128; i += 32)
+        stage_groups<129>(S.sh, S.perm, T[w], g0 + i / 16, S.n_groups,
+                          reinterpret_cast<uint32_t(*)[129]>(&W[w].tex[0][i]), W[w].raw);
+      bc1_encode_warp<128>(W[w], g0 * 16, gend * 16, reinterpret_cast<uint2*>(S.b1), S.sse1, S.sse0, nullptr);
+      __syncwarp();
     }
   }
 }
@@ -306,25 +302,20 @@ __global__ void __launch_bounds__(32 * BC7_WARPS, BC7_MIN_BLOCKS)
     k_batch7(const BatchSceneDev* __restrict__ scenes, int n_scenes, int64_t n_tiles, int schedule,
              int* __restrict__ counter) {
   __shared__ Bc7Warp W[BC7_WARPS];
-  __shared__ float s_scale[BC7_WARPS][16];
+  __shared__ StageScale T[BC7_WARPS];
   __shared__ uint8_t sq[12 * 256];
   for (int i = threadIdx.x; i < 12 * 256; i += blockDim.x) sq[i] = (&g_qtab[0][0])[i];
   __syncthreads();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int64_t it = 0;; it++) {
-    long long ti = 0;
-    if (lane == 0)
-      ti = (schedule == 0 || schedule == 3) ? (long long)((blockIdx.x + it * gridDim.x) * BC7_WARPS + w)
-                                            : (long long)atomicAdd(counter, 1);
-    ti = __shfl_sync(0xFFFFFFFFu, ti, 0);
+    const int64_t ti = claim_tile(schedule, it, w, lane, counter);
     if (ti >= n_tiles) break;
     const BatchSceneDev S = scene_of(scenes, n_scenes, ti);
     const int64_t gbeg = (ti - S.tile0) * S.tile_groups, gend = min(gbeg + (int64_t)S.tile_groups, S.work_groups);
-    if (lane < 16) s_scale[w][lane] = S.scales[lane];
+    stage_scales(T[w], S.scales);
     __syncwarp();
     for (int64_t g0 = gbeg; g0 < gend; g0 += 2) {
-      stage_groups<BC7_STRIDE, 1>(S.sh, S.perm, s_scale[w], g0, S.n_groups, W[w].tex, lane);
-      __syncwarp();
+      stage_groups<BC7_STRIDE, 1>(S.sh, S.perm, T[w], g0, S.n_groups, W[w].tex, reinterpret_cast<uint32_t*>(W[w].r));
       const int64_t blk = g0 * 16 + lane;
       const bool live = g0 + (lane >> 4) < gend;
       bc7_finish<32>(W[w], 0, live, blk, sq, reinterpret_cast<uint4*>(S.b7), S.sse7, nullptr);
@@ -336,13 +327,12 @@ __global__ void __launch_bounds__(32 * BC7_WARPS, BC7_MIN_BLOCKS)
 cudaError_t launch_batch_encode(int kind, const BatchSceneDev* scenes, int n_scenes, int64_t n_tiles, int schedule,
                                 int ctas_per_sm, int sm_count, int* counter, cudaStream_t st) {
   if (n_tiles <= 0 || n_scenes <= 0) return cudaSuccess;
-  // schedule 3: one claiming unit per tile, left to the hardware block scheduler; a BC7 CTA holds
-  // BC7_WARPS units, and a BC7 launch has BC7_MIN_BLOCKS CTAs (what one SM holds) per ctas_per_sm
-  const int64_t units = kind == 7 ? BC7_WARPS : 1;
-  const int64_t cta_tiles = ceil_div64(n_tiles, units);
+  // schedule 3: one claiming unit (a warp) per tile, left to the hardware block scheduler; a BC7 launch has
+  // BC7_MIN_BLOCKS CTAs (what one SM holds) per ctas_per_sm
+  const int64_t cta_tiles = ceil_div64(n_tiles, BC7_WARPS);
   int64_t grid = schedule == 3 ? cta_tiles
                                : (int64_t)(sm_count > 0 ? sm_count : gsc_sm_count()) *
-                                     (ctas_per_sm > 0 ? ctas_per_sm : (kind == 7 ? 1 : BC7_MIN_BLOCKS)) *
+                                     (ctas_per_sm > 0 ? ctas_per_sm : (kind == 7 ? 1 : 4)) *
                                      (kind == 7 ? BC7_MIN_BLOCKS : 1);
   if (grid > cta_tiles) grid = cta_tiles;
   if (grid > 0x7FFFFFFF) grid = 0x7FFFFFFF;
@@ -352,7 +342,7 @@ cudaError_t launch_batch_encode(int kind, const BatchSceneDev* scenes, int n_sce
   }
   gsc_count_launch();
   if (kind == 7) k_batch7<<<(int)grid, 32 * BC7_WARPS, 0, st>>>(scenes, n_scenes, n_tiles, schedule, counter);
-  else k_batch1<<<(int)grid, STAGE_THREADS, 0, st>>>(scenes, n_scenes, n_tiles, schedule, counter);
+  else k_batch1<<<(int)grid, 32 * BC7_WARPS, 0, st>>>(scenes, n_scenes, n_tiles, schedule, counter);
   return cudaGetLastError();
 }
 
@@ -377,17 +367,18 @@ __device__ __forceinline__ uint32_t mode1_err(const uint32_t* tex, int p, const 
   return (uint32_t)s;
 }
 
+#define M1_THREADS 128
 template <bool WARP>
-__global__ void __launch_bounds__(STAGE_THREADS) k_bc7_mode1(const uint8_t* __restrict__ texin, int64_t nblk,
+__global__ void __launch_bounds__(M1_THREADS) k_bc7_mode1(const uint8_t* __restrict__ texin, int64_t nblk,
                                                              uint32_t* __restrict__ sse_out,
                                                              int32_t* __restrict__ part_out) {
-  __shared__ uint32_t tex[STAGE_THREADS / 32][16][BC7_STRIDE];  // texel t of block 32 w + b at [w][t][b]
+  __shared__ uint32_t tex[M1_THREADS / 32][16][BC7_STRIDE];  // texel t of block 32 w + b at [w][t][b]
   __shared__ uint8_t sq[12 * 256];
   for (int i = threadIdx.x; i < 12 * 256; i += blockDim.x) sq[i] = (&g_qtab[0][0])[i];
   const int lt = threadIdx.x, w = lt >> 5, lane = lt & 31;
-  for (int64_t b0 = (int64_t)blockIdx.x * STAGE_THREADS; b0 < nblk; b0 += (int64_t)gridDim.x * STAGE_THREADS) {
+  for (int64_t b0 = (int64_t)blockIdx.x * M1_THREADS; b0 < nblk; b0 += (int64_t)gridDim.x * M1_THREADS) {
     __syncthreads();
-    for (int i = lt; i < STAGE_THREADS * 16; i += STAGE_THREADS) {
+    for (int i = lt; i < M1_THREADS * 16; i += M1_THREADS) {
       const int j = i / 16, t = i % 16;
       const int64_t blk = b0 + j;
       const uint8_t* p = texin + blk * 48 + 3 * t;
@@ -430,11 +421,11 @@ __global__ void __launch_bounds__(STAGE_THREADS) k_bc7_mode1(const uint8_t* __re
 cudaError_t launch_bc7_mode1(const uint8_t* tex, int64_t nblk, int warp, uint32_t* sse, int32_t* part, int sm_count,
                              cudaStream_t st) {
   if (nblk <= 0) return cudaSuccess;
-  int64_t g = ceil_div64(nblk, STAGE_THREADS);
+  int64_t g = ceil_div64(nblk, M1_THREADS);
   const int64_t cap = (int64_t)sm_count * 8;
   if (g > cap) g = cap;
   gsc_count_launch();
-  if (warp) k_bc7_mode1<true><<<(int)g, STAGE_THREADS, 0, st>>>(tex, nblk, sse, part);
-  else k_bc7_mode1<false><<<(int)g, STAGE_THREADS, 0, st>>>(tex, nblk, sse, part);
+  if (warp) k_bc7_mode1<true><<<(int)g, M1_THREADS, 0, st>>>(tex, nblk, sse, part);
+  else k_bc7_mode1<false><<<(int)g, M1_THREADS, 0, st>>>(tex, nblk, sse, part);
   return cudaGetLastError();
 }

@@ -1,56 +1,116 @@
-// stage.cuh -- layout-D tile staging shared by the group encoders (Sec. IV-B, Fig. SetupD).
+// stage.cuh -- layout-D staging shared by the group encoders (Sec. IV-B, Fig. SetupD): a warp turns two groups of
+// 16 slots into 32 blocks of 16 texels.
 //
-// A CTA of 128 threads owns 8 groups = 128 slots = 128 blocks. Thread i loads slot i
-// (group i / 16, texel i % 16): the Gaussian perm[slot] (a padding slot repeats the
-// group's last valid slot before it; none -> texel 128), its 48 floats as 12
-// 16-byte loads, quantises them (Sec. V-A) and scatters coefficient k into block
-// (group, k). Texels are packed r | g << 8 | b << 16 in smem tex[t][block]; the row
-// stride of 129 words keeps both the scatter and the per-block reads conflict-free.
+// Slot t of a group is the Gaussian perm[slot] (a padding slot repeats the group's last valid slot before it; none:
+// texel 128); its 48 floats are quantised (Sec. V-A) and coefficient k goes to texel t of block (group, k), packed
+// r | g << 8 | b << 16 at tex[t][block].
+//
+// The rows lie anywhere in memory, so the time is that of the reads: twelve neighbouring lanes read one row of 192
+// bytes in 16-byte pieces, whole sectors at a time. One lane per row instead read half a sector per request and
+// found the other half gone from L1: 3M Gaussians in 390 us, against 170 us. The quantised bytes cross over
+// in shared memory; the odd row strides keep every access but the pieces' own free of conflicts.
 #pragma once
 #include "gsc_internal.cuh"
 
-#define STAGE_GROUPS 8
-#define STAGE_THREADS 128
-#define STAGE_STRIDE 129
+#define STAGE_RAW (32 * 13)  // words of crossing space per warp
 
-// i: the thread's index inside its staging unit of 128 threads, or of one warp (two groups); a multiple
-// of 32 apart from threadIdx.x, so the warp-level ballots below see the same lanes. STRIDE: words between
-// texel rows, one more than the unit's blocks. STEPS: steps of four coefficients unrolled (4: all loads in
-// flight together; 1: a quarter of the code).
+// The scales spread over a row's 48 floats, and their reciprocals.
+struct StageScale {
+  float4 s[12], r[12];
+  int fast;  // every scale is in [2^-60, 2^60]
+};
+
+// by one warp
+__device__ __forceinline__ void stage_scales(StageScale& T, const float* __restrict__ scales) {
+  const int lane = threadIdx.x & 31;
+  const float s = scales[lane & 15], r = __frcp_rn(s);
+  const bool fast = __all_sync(0xFFFFFFFFu, s >= 0x1p-60f && s <= 0x1p60f);
+  if (lane < 16)
+    for (int c = 0; c < 3; c++) {
+      reinterpret_cast<float*>(T.s)[3 * lane + c] = s;
+      reinterpret_cast<float*>(T.r)[3 * lane + c] = r;
+    }
+  if (lane == 0) T.fast = fast;
+}
+
+// gsc_quant1 without the divide, r = RN(1 / s): the code is the low byte of the result. Beyond +-0.503 s and 0.499 s
+// the code is 0 or 255 (x / s * 255 is past -128.2 or 127.2 and rounds to -128 or 127 at least), so x is clamped there
+// (NaN to the lower end, as there). The quotient is rounded correctly by Markstein's correction (IBM J. Res. Dev. 34,
+// 1990): q0 = RN(x r) is off by at most 1.5 ulp; a first residual step brings that below one, where the second residual
+// is exact and RN(q + r e) = RN(x / s). Residuals that underflow belong to |x| < 2^-78, whose code is 128 in any
+// case. Adding 1.5 * 2^23 + 128 rounds to an integer, ties to even, as rint does.
+__device__ __forceinline__ uint32_t stage_quant(float x, float s, float r) {
+  x = fminf(fmaxf(x, s * -0.503f), s * 0.499f);
+  float q = __fmul_rn(x, r);
+  q = __fmaf_rn(__fmaf_rn(-q, s, x), r, q);
+  q = __fmaf_rn(__fmaf_rn(-q, s, x), r, q);
+  return __float_as_uint(__fadd_rn(__fmul_rn(q, 255.0f), 12583040.0f));
+}
+__device__ __forceinline__ uint32_t stage_quant4(float4 x, float4 s, float4 r) {
+  const uint32_t lo = __byte_perm(stage_quant(x.x, s.x, r.x), stage_quant(x.y, s.y, r.y), 0x0040);
+  const uint32_t hi = __byte_perm(stage_quant(x.z, s.z, r.z), stage_quant(x.w, s.w, r.w), 0x0040);
+  return __byte_perm(lo, hi, 0x5410);
+}
+
+// By one warp: groups g0 and g0 + 1 (those below n_groups) into the 32 columns of tex. STRIDE: words between texel
+// rows, one more than a multiple of 32. raw: STAGE_RAW words. STEPS: eighths of rows read ahead, times 8 rows
+// (4: all in flight together; 1: a quarter of the code).
 template <int STRIDE, int STEPS = 4>
 __device__ __forceinline__ void stage_groups(const float* __restrict__ sh, const int32_t* __restrict__ perm,
-                                             const float* s_scale, int64_t g0, int64_t n_groups,
-                                             uint32_t (*tex)[STRIDE], int i) {
-  const int lg = i >> 4, t = i & 15;
-  const int64_t g = g0 + lg;
-  const bool live = g < n_groups;
-  int32_t o = live ? __ldg(perm + g * 16 + t) : -1;
+                                             const StageScale& T, int64_t g0, int64_t n_groups,
+                                             uint32_t (*tex)[STRIDE], uint32_t* raw) {
+  int lane = threadIdx.x & 31;
+  asm volatile("" : "+r"(lane));  // what derives from it is not kept in registers between calls
+  const int t = lane & 15;
+  const int64_t g = g0 + (lane >> 4);
+  const int32_t o = g < n_groups ? __ldg(perm + g * 16 + t) : -1;
   // last valid slot at or before t inside this half-warp's group
-  const unsigned half = 0xFFFFu << (threadIdx.x & 16);
-  unsigned valid = __ballot_sync(0xFFFFFFFFu, o >= 0) & half;
-  unsigned upto = valid & (0xFFFFFFFFu >> (31 - (threadIdx.x & 31)));
-  int src_lane = upto ? 31 - __clz(upto) : -1;
-  int32_t src = __shfl_sync(0xFFFFFFFFu, o, src_lane < 0 ? (threadIdx.x & 31) : src_lane);
-  if (src_lane < 0) src = -1;
-  const int col = lg * 16;
-  if (src < 0) {
+  const unsigned upto = __ballot_sync(0xFFFFFFFFu, o >= 0) & (0xFFFFu << (lane & 16)) & (0xFFFFFFFFu >> (31 - lane));
+  const int32_t got = __shfl_sync(0xFFFFFFFFu, o, upto ? 31 - __clz(upto) : lane);
+  const int32_t src = upto ? got : -1;
+  if (T.fast) {
+    // piece 32 b + lane of the eight rows 8 a .. 8 a + 7
+    const int p0 = lane % 12, p1 = (lane + 8) % 12, p2 = (lane + 4) % 12;
+    const int r0 = lane / 12, r1 = (lane + 32) / 12, r2 = (lane + 64) / 12;
+#pragma unroll 1
+    for (int a0 = 0; a0 < 4; a0 += STEPS) {
+      float4 x[STEPS][3];
 #pragma unroll
-    for (int k = 0; k < 16; k++) tex[t][col + k] = 128u | (128u << 8) | (128u << 16);
-    return;
-  }
-  const float4* p = reinterpret_cast<const float4*>(sh + (int64_t)src * 48);
-  // four coefficients (three 16-byte loads) per step
-#pragma unroll STEPS
-  for (int j = 0; j < 4; j++) {
-    const float4 a = __ldg(p + 3 * j), b = __ldg(p + 3 * j + 1), c = __ldg(p + 3 * j + 2);
-    const float v[12] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y, c.z, c.w};
+      for (int a = 0; a < STEPS; a++)
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-      const float s = s_scale[4 * j + k];
-      const uint32_t r = gsc_quant1(v[3 * k + 0], s), g = gsc_quant1(v[3 * k + 1], s), b8 = gsc_quant1(v[3 * k + 2], s);
-      tex[t][col + 4 * j + k] = r | (g << 8) | (b8 << 16);
+        for (int b = 0; b < 3; b++) {
+          const int p = b == 0 ? p0 : b == 1 ? p1 : p2, row = 8 * (a0 + a) + (b == 0 ? r0 : b == 1 ? r1 : r2);
+          const int32_t from = __shfl_sync(0xFFFFFFFFu, src, row);
+          x[a][b] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          if (from >= 0) x[a][b] = __ldg(reinterpret_cast<const float4*>(sh + (int64_t)from * 48) + p);
+        }
+#pragma unroll
+      for (int b = 0; b < 3; b++) {
+        const int p = b == 0 ? p0 : b == 1 ? p1 : p2, row = 8 * a0 + (b == 0 ? r0 : b == 1 ? r1 : r2);
+        const float4 s = T.s[p], r = T.r[p];
+#pragma unroll
+        for (int a = 0; a < STEPS; a++) raw[(row + 8 * a) * 13 + p] = stage_quant4(x[a][b], s, r);
+      }
     }
+  } else {
+    uint8_t* q = reinterpret_cast<uint8_t*>(raw + lane * 13);
+#pragma unroll 1
+    for (int e = 0; e < 48; e++)
+      q[e] = src < 0 ? (uint8_t)128
+                     : (uint8_t)gsc_quant1(__ldg(sh + (int64_t)src * 48 + e), reinterpret_cast<const float*>(T.s)[e]);
   }
+  __syncwarp();
+  const uint32_t* q = raw + lane * 13;
+  const int col = lane & 16;
+#pragma unroll
+  for (int j = 0; j < 4; j++) {
+    const uint32_t a = q[3 * j], b = q[3 * j + 1], c = q[3 * j + 2];
+    tex[t][col + 4 * j] = a & 0xFFFFFFu;
+    tex[t][col + 4 * j + 1] = __funnelshift_r(a, b, 24) & 0xFFFFFFu;
+    tex[t][col + 4 * j + 2] = __funnelshift_r(b, c, 16) & 0xFFFFFFu;
+    tex[t][col + 4 * j + 3] = c >> 8;
+  }
+  __syncwarp();
 }
 
 __device__ __forceinline__ int tex_r(uint32_t v) { return v & 255; }
