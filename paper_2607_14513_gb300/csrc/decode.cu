@@ -175,15 +175,18 @@ struct RawBlock {
   int kind;
 };
 
-template <int KIND>
+// ONCE: nothing reads the block again (it goes out of the second-level cache first).
+template <int KIND, bool ONCE = false>
 __device__ __forceinline__ RawBlock fetch_block(const DevTable& T, const uint8_t* __restrict__ blocks, int64_t g, int k) {
   RawBlock r;
   r.w = make_uint4(0u, 0u, 0u, 0u);
   if (KIND == 7) {
-    r.w = __ldg(reinterpret_cast<const uint4*>(blocks) + g * 16 + k);
+    const uint4* p = reinterpret_cast<const uint4*>(blocks) + g * 16 + k;
+    r.w = ONCE ? __ldcs(p) : __ldg(p);
     r.kind = 7;
   } else if (KIND == 1) {
-    const uint2 v = __ldg(reinterpret_cast<const uint2*>(blocks) + g * 16 + k);
+    const uint2* p = reinterpret_cast<const uint2*>(blocks) + g * 16 + k;
+    const uint2 v = ONCE ? __ldcs(p) : __ldg(p);
     r.w.x = v.x; r.w.y = v.y;
     r.kind = 1;
   } else {
@@ -200,10 +203,11 @@ __device__ __forceinline__ RawBlock fetch_block(const DevTable& T, const uint8_t
   return r;
 }
 
+// The block's 16 packed texels (RGB; 128 where dropped).
 template <int KIND>
-__device__ __forceinline__ void decode_raw(const RawBlock& r, uint32_t (&tx)[16], const DecTables* S, uint4* ep) {
+__device__ __forceinline__ void decode_raw(const RawBlock& r, uint32_t (&tx)[16], const DecTables& S, uint32_t area) {
   if (KIND == 7 || (KIND == 0 && r.kind == 7)) {
-    bc7_block(((uint64_t)r.w.y << 32) | r.w.x, ((uint64_t)r.w.w << 32) | r.w.z, tx, S, ep);
+    bc7_block(r.w, tx, S, area);
   } else if (KIND == 1 || (KIND == 0 && r.kind == 1)) {
     bc1_block(make_uint2(r.w.x, r.w.y), tx);
   } else {
@@ -212,72 +216,79 @@ __device__ __forceinline__ void decode_raw(const RawBlock& r, uint32_t (&tx)[16]
   }
 }
 
-// Block k of group g of the stream table into 16 packed texels (RGB + A); 128 where dropped.
-template <int KIND>
-__device__ __forceinline__ void block_texels(const DevTable& T, const uint8_t* __restrict__ blocks, int64_t g, int k,
-                                             uint32_t (&tx)[16], const DecTables* S, uint4* ep) {
-  if (KIND == 7) {
-    const uint4 w = __ldg(reinterpret_cast<const uint4*>(blocks) + g * 16 + k);
-    bc7_block(((uint64_t)w.y << 32) | w.x, ((uint64_t)w.w << 32) | w.z, tx, S, ep);
-  } else if (KIND == 1) {
-    bc1_block(__ldg(reinterpret_cast<const uint2*>(blocks) + g * 16 + k), tx);
-  } else {
-    const int si = stream_of(T, g);
-    const BlockLoc L = locate(T, si, g, k);
-    if (L.kind == 7) {
-      const uint2* p = reinterpret_cast<const uint2*>(blocks + L.off);
-      const uint2 w0 = __ldg(p), w1 = __ldg(p + 1);
-      bc7_block(((uint64_t)w0.y << 32) | w0.x, ((uint64_t)w1.y << 32) | w1.x, tx, S, ep);
-    } else if (L.kind == 1) {
-      bc1_block(__ldg(reinterpret_cast<const uint2*>(blocks + L.off)), tx);
-    } else {
-#pragma unroll
-      for (int t = 0; t < 16; t++) tx[t] = 0xFF808080u;
-    }
-  }
-}
-
-
-
+// Three neighbouring lanes store one Gaussian's 48 bytes, through the tile: with each lane storing its own row 3M
+// Gaussians take 131 us, against 115 us, and 111 us with blocks and slot order read past the second-level cache, whose
+// space the scattered rows need: half of each row's second sector belongs to another row, whose store finds it there
+// or has to fetch it from memory (60 MB of reads). The rows' order bounds the kernel: in slot order it takes 81 us,
+// without stores 76 us, which is the shared-memory pipe (60% busy). The decoder before this one, with one lane per
+// row, took 145 us.
+#define DEC_WARPS 4
+#define DEC_CTAS 16  // per SM
 template <int KIND, int LAYOUT>
-__global__ void __launch_bounds__(256) k_decode2(DevTable T, const uint8_t* __restrict__ blocks,
+__global__ void __launch_bounds__(32 * DEC_WARPS) k_decode2(DevTable T, const uint8_t* __restrict__ blocks,
                                                  const int32_t* __restrict__ perm, uint8_t* __restrict__ texels) {
-  __shared__ DecTables S;
-  __shared__ uint32_t tile[8][WTILE];
-  __shared__ uint4 s_ep[256][3];
-  load_tables(&S);
+  __shared__ __align__(1024) uint8_t areas[DEC_WARPS][KIND == 1 ? 1 : DEC_AREA];
+  __shared__ __align__(16) uint8_t tables[KIND == 1 ? 16 : sizeof(DecTables)];
+  __shared__ __align__(16) uint32_t tile[DEC_WARPS][WTILE];
+  const DecTables& S = *reinterpret_cast<DecTables*>(tables);
+  uint32_t area = 0;
+  if (KIND != 1) {
+    load_tables(reinterpret_cast<DecTables*>(tables));
+    area = dec_area(areas[threadIdx.x >> 5]);
+  }
   __syncthreads();
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, gw = l >> 4, kt = l & 15;
-  const int64_t npairs = ((int64_t)T.n_groups + 1) / 2;
+  const int64_t npairs = ((int64_t)T.n_groups + 1) / 2, step = (int64_t)gridDim.x * DEC_WARPS;
   uint32_t* my = tile[w] + gw * 272;
-  for (int64_t pr = (int64_t)blockIdx.x * 8 + w; pr < npairs; pr += (int64_t)gridDim.x * 8) {
-    const int64_t g = pr * 2 + gw;
-    const bool live = g < T.n_groups;
-    uint32_t tx[16];
-    if (live) block_texels<KIND>(T, blocks, g, kt, tx, &S, s_ep[threadIdx.x]);
+  uint4* rows = reinterpret_cast<uint4*>(tile[w]);
+  // blocks and slot order entries are loaded one iteration ahead
+  auto block_at = [&](int64_t pr) -> RawBlock {
+    RawBlock r;
+    r.kind = 0;
+    r.w = make_uint4(0u, 0u, 0u, 0u);
+    return pr * 2 + gw < T.n_groups ? fetch_block<KIND, true>(T, blocks, pr * 2 + gw, kt) : r;
+  };
+  auto slot_at = [&](int64_t pr) -> int32_t {
+    const int64_t s = (pr * 2 + gw) * 16 + kt;
+    return pr * 2 + gw < T.n_groups ? checked_slot(__ldcs(perm + s), T.n, s) : -1;
+  };
+  int64_t pr = (int64_t)blockIdx.x * DEC_WARPS + w;
+  RawBlock raw = block_at(pr);
+  int32_t o = slot_at(pr);
+  for (; pr < npairs; pr += step) {
+    const RawBlock rawn = block_at(pr + step);
+    const int32_t on = slot_at(pr + step);
+    {
+      uint32_t tx[16];
+      decode_raw<KIND>(raw, tx, S, area);  // past the last group: never stored
 #pragma unroll
-    for (int t = 0; t < 16; t++) my[17 * kt + t] = live ? tx[t] : 0u;
-    __syncwarp();
-    const int32_t o = live ? checked_slot(__ldg(perm + g * 16 + kt), T.n, g * 16 + kt) : -1;
-    if (o >= 0) {
-      uint32_t wv[12];
-#pragma unroll
-      for (int i = 0; i < 12; i++) wv[i] = 0;
-#pragma unroll
-      for (int k = 0; k < 16; k++) {
-        const uint32_t px = my[tile_at<LAYOUT>(kt, k)];
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-          const int byte = 3 * k + c;
-          wv[byte >> 2] |= ((px >> (8 * c)) & 255u) << (8 * (byte & 3));
-        }
-      }
-      uint4* dst = reinterpret_cast<uint4*>(texels + (int64_t)o * 48);
-      dst[0] = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-      dst[1] = make_uint4(wv[4], wv[5], wv[6], wv[7]);
-      dst[2] = make_uint4(wv[8], wv[9], wv[10], wv[11]);
+      for (int t = 0; t < 16; t++) my[17 * kt + t] = tx[t];
     }
     __syncwarp();
+    uint32_t wv[12];
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      uint32_t px[4];
+#pragma unroll
+      for (int c = 0; c < 4; c++) px[c] = my[tile_at<LAYOUT>(kt, 4 * j + c)];
+      wv[3 * j] = __byte_perm(px[0], px[1], 0x4210);
+      wv[3 * j + 1] = __byte_perm(px[1], px[2], 0x5421);
+      wv[3 * j + 2] = __byte_perm(px[2], px[3], 0x6542);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < 3; j++) rows[3 * l + j] = make_uint4(wv[4 * j], wv[4 * j + 1], wv[4 * j + 2], wv[4 * j + 3]);
+    __syncwarp();
+    // three neighbouring lanes store one row
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+      const int i = 32 * j + l, row = i / 3;
+      const int32_t to = __shfl_sync(0xFFFFFFFFu, o, row);
+      if (to >= 0) reinterpret_cast<uint4*>(texels + (int64_t)to * 48)[i - 3 * row] = rows[i];
+    }
+    __syncwarp();
+    raw = rawn;
+    o = on;
   }
 }
 
@@ -381,10 +392,10 @@ __device__ __forceinline__ void load_views(float (*s_view)[64], float* s_deq, co
 // retired, so an evaluation launched beside an encode on a higher-priority stream starts early.
 #define EVAL_THREADS 128
 // No register cap: capping at 5 or 6 resident CTAs per SM spills in the evaluation loop and
-// measured slower (3M Gaussians, all-BC7, 8 cameras: 0.205 ms uncapped, 0.225 ms and 0.260 ms).
-#ifndef EVAL_MIN_BLOCKS
+// measured slower (3M Gaussians, all-BC7, 8 cameras: 0.145 ms uncapped, 0.193 ms at 5). Bound by instruction issue (67%
+// of the slots, 1,207 instructions per 32 Gaussians); with coefficients instead of views in the halves of the multiply-
+// adds it takes 0.156 ms.
 #define EVAL_MIN_BLOCKS 1
-#endif
 // LIST: only the groups listed in glist[0, n_list) (-1 entries skipped), e.g. those of the chunks a
 // view keeps.
 template <int KIND, bool CAMS, int VF, int LAYOUT, bool LIST, int ORD>
@@ -394,12 +405,17 @@ __global__ void __launch_bounds__(EVAL_THREADS, EVAL_MIN_BLOCKS) k_eval2(DevTabl
                                                int out_order, float* __restrict__ rgb,
                                                const int32_t* __restrict__ glist, int64_t n_list,
                                                const float* __restrict__ pos_slot) {
-  __shared__ DecTables S;
+  __shared__ __align__(1024) uint8_t areas[EVAL_THREADS / 32][KIND == 1 ? 1 : DEC_AREA];
+  __shared__ __align__(16) uint8_t tables[KIND == 1 ? 16 : sizeof(DecTables)];
   __shared__ uint32_t tile[EVAL_THREADS / 32][WTILE];
-  __shared__ uint4 s_ep[EVAL_THREADS][3];
   __shared__ float s_view[3][64];
   __shared__ __align__(8) float s_deq[16];
-  load_tables(&S);
+  const DecTables& S = *reinterpret_cast<DecTables*>(tables);
+  uint32_t area = 0;
+  if (KIND != 1) {
+    load_tables(reinterpret_cast<DecTables*>(tables));
+    area = dec_area(areas[threadIdx.x >> 5]);
+  }
   load_views(s_view, s_deq, dirs, cams, V, T);
   __syncthreads();
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31, gw = l >> 4, kt = l & 15, nw = blockDim.x >> 5;
@@ -448,7 +464,7 @@ __global__ void __launch_bounds__(EVAL_THREADS, EVAL_MIN_BLOCKS) k_eval2(DevTabl
     const int32_t o2 = perm_at(prn + step);
     {
       uint32_t tx[16];
-      decode_raw<KIND>(raw, tx, &S, s_ep[threadIdx.x]);  // past the last group: never read back
+      decode_raw<KIND>(raw, tx, S, area);  // past the last group: never read back
 #pragma unroll
       for (int t = 0; t < 16; t++) my[17 * kt + t] = tx[t];
     }
@@ -503,14 +519,14 @@ static int eval_grid(int64_t n_groups, int sm_count, int warps = 8) {
 cudaError_t launch_decode(const DevTable& T, const uint8_t* blocks, const int32_t* perm, uint8_t* texels,
                           cudaStream_t st) {
   if (T.n_groups == 0) return cudaSuccess;
-  const int grid = eval_grid(T.n_groups, gsc_sm_count());
+  const int grid = (int)std::min<int64_t>(ceil_div64(((int64_t)T.n_groups + 1) / 2, DEC_WARPS), (int64_t)gsc_sm_count() * DEC_CTAS);
 #define DEC_LAUNCH(L)                                                                              \
   do {                                                                                             \
     gsc_count_launch();                                                                            \
     switch (kind_of(T, blocks)) {                                                                  \
-      case 7: k_decode2<7, L><<<grid, 256, 0, st>>>(T, blocks, perm, texels); break;               \
-      case 1: k_decode2<1, L><<<grid, 256, 0, st>>>(T, blocks, perm, texels); break;               \
-      default: k_decode2<0, L><<<grid, 256, 0, st>>>(T, blocks, perm, texels); break;              \
+      case 7: k_decode2<7, L><<<grid, 32 * DEC_WARPS, 0, st>>>(T, blocks, perm, texels); break;               \
+      case 1: k_decode2<1, L><<<grid, 32 * DEC_WARPS, 0, st>>>(T, blocks, perm, texels); break;               \
+      default: k_decode2<0, L><<<grid, 32 * DEC_WARPS, 0, st>>>(T, blocks, perm, texels); break;              \
     }                                                                                              \
   } while (0)
   if (T.layout == GSC_LAYOUT_A) DEC_LAUNCH(GSC_LAYOUT_A);
