@@ -425,7 +425,7 @@ __device__ __forceinline__ void block_sort(uint32_t* s_key, V* s_val, uint32_t (
       val[r] = i < count ? s_val[i] : (V)0;
     }
     auto digit = [&](int r) { return first + 32 * r < count ? (key[r] >> (8 * p)) & 255u : 256u; };
-    const uint32_t mine = rank_digits<WARPS, ITEMS, 8>(digit, rank, s_cnt);
+    const uint32_t mine = rank_digits<WARPS, ITEMS, 8>(digit, [&](int r, uint32_t x) { rank[r] = x; }, s_cnt);
     const uint64_t start = prefix256(threadIdx.x < 256 ? mine : 0u, s_scan);
     if (threadIdx.x < 256) s_start[threadIdx.x] = (uint32_t)start;
     __syncthreads();

@@ -1,9 +1,11 @@
 // sort.cu -- device-wide stable LSD radix sort of (key, u32 value) pairs, 8-bit digits, and the exclusive scan.
 //
 // A pass is three kernels over tiles of 4096 pairs: digit counts per tile, a scan of each digit's row of counts
-// (one CTA per digit), and the tiles ranked, sorted in shared memory and written out in runs: 9 + 3 + 33 us at 3M
+// (one CTA per digit), and the tiles ranked, sorted in shared memory and written out in runs: 9 + 3 + 24 us at 3M
 // pairs of 32-bit keys (one GB300, each kernel alone with cold caches), against 12 + 15 + 58 us with a three-kernel
-// scan and three CTA barriers per 32 items in the scatter. No kernel waits for another CTA: chaining the tiles in
+// scan and three CTA barriers per 32 items in the scatter. The scatter is bound by latency: with the values read only
+// after the keys had been placed, and half the items in flight, it took 33 us, and 30M pairs of 16-bit keys 246 us
+// against 149 us; four CTAs per SM instead of three take as long. No kernel waits for another CTA: chaining the tiles in
 // one kernel (decoupled look-back) took 41 us per pass with two resident CTAs per SM and 470 us with four, when
 // most of the machine polled. 32-bit keys where the caller's fit.
 #include "sort.cuh"
@@ -176,12 +178,12 @@ __global__ void __launch_bounds__(256) k_rs_rows(uint32_t* __restrict__ counts, 
 
 // vin = nullptr: values are the input positions; kout = nullptr: the sorted keys are not wanted
 template <class K, int BITS>
-__global__ void __launch_bounds__(RS_THREADS, sizeof(K) <= 4 ? 4 : 3)
+__global__ void __launch_bounds__(RS_THREADS, 3)
     k_rs_scatter(const K* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t n, int shift,
                  const uint32_t* __restrict__ total, const uint32_t* __restrict__ counts, K* __restrict__ kout,
                  uint32_t* __restrict__ vout) {
-  __shared__ uint64_t s_items[RS_TILE * (sizeof(K) > 4 ? sizeof(K) : 4) / 8];
-  K* s_item = reinterpret_cast<K*>(s_items);  // the sorted keys, then the sorted values
+  __shared__ K s_key[RS_TILE];
+  __shared__ uint32_t s_val[RS_TILE];
   __shared__ uint32_t s_cnt[RS_WARPS][256];
   __shared__ uint32_t s_start[256], s_base[256];
   __shared__ uint64_t s_scan[8];
@@ -189,14 +191,23 @@ __global__ void __launch_bounds__(RS_THREADS, sizeof(K) <= 4 ? 4 : 3)
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int64_t base = (int64_t)blockIdx.x * RS_TILE;
   const int count = (int)min((int64_t)RS_TILE, n - base);
-  const uint32_t before = counts[(int64_t)t * gridDim.x + blockIdx.x], all = total[t];
-  K key[RS_ITEMS];
-  uint32_t rank[RS_ITEMS];
+  constexpr bool PACK = sizeof(K) == 2;  // the key's bits above its item's rank
+  K key[PACK ? 1 : RS_ITEMS];
+  uint32_t val[RS_ITEMS], rank[RS_ITEMS];
   const int first = w * (RS_ITEMS * 32) + lane;  // the thread's items: first + 32 r
 #pragma unroll
-  for (int r = 0; r < RS_ITEMS; r++) key[r] = first + 32 * r < count ? kin[base + first + 32 * r] : (K)0;
-  auto digit = [&](int r) { return first + 32 * r < count ? (uint32_t)(key[r] >> shift) & mask : 256u; };
-  const uint32_t mine = rank_digits<RS_WARPS, RS_ITEMS, BITS>(digit, rank, s_cnt);
+  for (int r = 0; r < RS_ITEMS; r++) {
+    const K k = first + 32 * r < count ? kin[base + first + 32 * r] : (K)0;
+    if (PACK) rank[r] = (uint32_t)k << 16;
+    else key[r] = k;
+  }
+  const uint32_t before = counts[(int64_t)t * gridDim.x + blockIdx.x], all = total[t];
+#pragma unroll
+  for (int r = 0; r < RS_ITEMS; r++)
+    val[r] = !vin ? (uint32_t)(base + first + 32 * r) : first + 32 * r < count ? __ldg(vin + base + first + 32 * r) : 0u;
+  auto key_of = [&](int r) { return PACK ? (K)(rank[r] >> 16) : key[PACK ? 0 : r]; };
+  auto digit = [&](int r) { return first + 32 * r < count ? (uint32_t)(key_of(r) >> shift) & mask : 256u; };
+  const uint32_t mine = rank_digits<RS_WARPS, RS_ITEMS, BITS>(digit, [&](int r, uint32_t x) { rank[r] = PACK ? rank[r] | x : x; }, s_cnt);
   // where digit t starts in the output and in the tile
   const uint64_t both = prefix256(((uint64_t)all << 16) | mine, s_scan);
   const uint32_t start = (uint32_t)(both & 0xFFFFu);
@@ -206,30 +217,19 @@ __global__ void __launch_bounds__(RS_THREADS, sizeof(K) <= 4 ? 4 : 3)
 #pragma unroll
   for (int r = 0; r < RS_ITEMS; r++)
     if (first + 32 * r < count) {
-      const uint32_t d = digit(r);
-      rank[r] += s_start[d] + s_cnt[w][d];  // now the place in the sorted tile
-      s_item[rank[r]] = key[r];
+      const uint32_t d = digit(r), at = (PACK ? rank[r] & 0xFFFFu : rank[r]) + s_start[d] + s_cnt[w][d];  // the place in the sorted tile
+      s_key[at] = key_of(r);
+      s_val[at] = val[r];
     }
   __syncthreads();
-  uint32_t dst[RS_ITEMS];
 #pragma unroll
   for (int r = 0; r < RS_ITEMS; r++) {
     const int i = r * RS_THREADS + t;
     if (i >= count) continue;
-    const K k = s_item[i];
-    dst[r] = s_base[(uint32_t)(k >> shift) & mask] + (uint32_t)i;
-    if (kout) kout[dst[r]] = k;
-  }
-  __syncthreads();
-  uint32_t* s_val = reinterpret_cast<uint32_t*>(s_item);
-#pragma unroll
-  for (int r = 0; r < RS_ITEMS; r++)
-    if (first + 32 * r < count) s_val[rank[r]] = vin ? __ldg(vin + base + first + 32 * r) : (uint32_t)(base + first + 32 * r);
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < RS_ITEMS; r++) {
-    const int i = r * RS_THREADS + t;
-    if (i < count) vout[dst[r]] = s_val[i];
+    const K k = s_key[i];
+    const uint32_t dst = s_base[(uint32_t)(k >> shift) & mask] + (uint32_t)i;
+    if (kout) kout[dst] = k;
+    vout[dst] = s_val[i];
   }
 }
 

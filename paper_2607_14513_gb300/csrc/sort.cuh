@@ -23,13 +23,13 @@ __device__ __forceinline__ uint64_t prefix256(uint64_t v, uint64_t* s) {
 }
 
 // Stable ranks of a CTA's items by a digit of BITS (at most 8) bits. Warp w holds ITEMS * 32 consecutive items, item r of lane l
-// being r * 32 + l of them; digit(r) = 256 for an item past the end. On return rank[r] is the item's position
-// among its warp's items of the same digit, and cnt[w][d] the number of items of digit d in the warps before w;
+// being r * 32 + l of them; digit(r) = 256 for an item past the end. put(r, rank) takes the item's position
+// among its warp's items of the same digit; on return cnt[w][d] is the number of items of digit d in the warps before w;
 // the total per digit is returned to thread d < 256. cnt has WARPS rows. A round's peers come from BITS ballots
 // (a match instruction took several times as long on digits that mostly differ), and its leaders take their
 // places with one shared-memory addition each: rounds wait neither for one another nor for a barrier.
-template <int WARPS, int ITEMS, int BITS, class Digit>
-__device__ __forceinline__ uint32_t rank_digits(Digit digit, uint32_t (&rank)[ITEMS], uint32_t (*cnt)[256]) {
+template <int WARPS, int ITEMS, int BITS, class Digit, class Put>
+__device__ __forceinline__ uint32_t rank_digits(Digit digit, Put put, uint32_t (*cnt)[256]) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t below = (1u << lane) - 1u;
 #pragma unroll
@@ -48,7 +48,7 @@ __device__ __forceinline__ uint32_t rank_digits(Digit digit, uint32_t (&rank)[IT
     const uint32_t before = __popc(peers & below);
     uint32_t old = 0u;
     if (live && before == 0u) old = atomicAdd(&cnt[w][d], (uint32_t)__popc(peers));
-    rank[r] = __shfl_sync(0xFFFFFFFFu, old, live ? __ffs(peers) - 1 : lane) + before;
+    put(r, __shfl_sync(0xFFFFFFFFu, old, live ? __ffs(peers) - 1 : lane) + before);
   }
   __syncthreads();
   uint32_t sum = 0;
