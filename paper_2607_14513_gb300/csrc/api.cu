@@ -257,6 +257,15 @@ extern "C" const char* gsc_status_string(gsc_status s) {
 
 extern "C" gsc_status gsc_ctx_create(gsc_ctx** out, int device) { return ctx_new(device, true, out); }
 
+static void ctx_free(gsc_ctx* c) {
+  if (c->d_status) cudaFree(c->d_status);
+  if (c->h_pinned) cudaFreeHost(c->h_pinned);
+  if (c->side_join) cudaEventDestroy(c->side_join);
+  if (c->side_fork) cudaEventDestroy(c->side_fork);
+  if (c->side) cudaStreamDestroy(c->side);
+  free(c);
+}
+
 gsc_status ctx_new(int device, bool init_tables, gsc_ctx** out) {
   if (!out) return GSC_ERR_INVALID_ARG;
   *out = nullptr;
@@ -278,6 +287,9 @@ gsc_status ctx_new(int device, bool init_tables, gsc_ctx** out) {
   if (e == cudaSuccess) { c->d_diag = c->d_status + 1; e = cudaMemset(c->d_status, 0, 2 * sizeof(int)); }
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_pinned, PINNED_BYTES);
   c->h_pinned_bytes = PINNED_BYTES;
+  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->side_fork, cudaEventDisableTiming);
+  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->side_join, cudaEventDisableTiming);
   if (init_tables) {
     if (e == cudaSuccess) e = bc1_init_tables();
     if (e == cudaSuccess) e = bc7_init_tables();
@@ -286,9 +298,7 @@ gsc_status ctx_new(int device, bool init_tables, gsc_ctx** out) {
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
   }
   if (e != cudaSuccess) {
-    if (c->d_status) cudaFree(c->d_status);
-    if (c->h_pinned) cudaFreeHost(c->h_pinned);
-    free(c);
+    ctx_free(c);
     return GSC_ERR_CUDA;
   }
   *out = c;
@@ -302,9 +312,7 @@ extern "C" gsc_status gsc_ctx_destroy(gsc_ctx* c) {
   free(c->recs);
   cudaDeviceSynchronize();
   tex_cache_free(c);
-  if (c->d_status) cudaFree(c->d_status);
-  if (c->h_pinned) cudaFreeHost(c->h_pinned);
-  free(c);
+  ctx_free(c);
   return GSC_OK;
 }
 

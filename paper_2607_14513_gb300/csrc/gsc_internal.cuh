@@ -35,6 +35,8 @@ struct gsc_ctx {
   int* d_diag;          // where it happened (kernel-defined)
   void* h_pinned;       // small pinned host buffer for table read-back
   size_t h_pinned_bytes;
+  cudaStream_t side;    // for the half of a plan that runs beside the other
+  cudaEvent_t side_fork, side_join;
 };
 
 #define GSC_CUDA(call)                                   \

@@ -61,3 +61,25 @@ def test_scales_at_other_quantiles(ctx, O, n, permille):
     _, scales = gsc.gsc_plan_reorder(ctx, None, torch.from_numpy(sh).cuda(), sort=0, permille=permille)
     ctx.sync()
     assert np.array_equal(scales.cpu().numpy(), O.scales(sh, permille))
+
+
+@pytest.mark.parametrize("n", [4096, 20_001])
+def test_plan_captured_and_eager_agree(ctx, n):
+    """A captured plan (one stream) replays to what the eager plan (two streams) gives, also with an eager plan of the
+    same context enqueued while the capture is open."""
+    from paper_2607_14513_gb300 import gsc
+    sc = _scene(n, "random", 5)
+    pos, sh = torch.from_numpy(sc.pos).cuda(), torch.from_numpy(sc.sh).cuda()
+    ws = [ctx.workspace(n) for _ in range(2)]
+    want = gsc.gsc_plan_reorder(ctx, pos, sh, ws=ws[0])
+    torch.cuda.synchronize()
+    other, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, capture_error_mode="thread_local"):
+        got = gsc.gsc_plan_reorder(ctx, pos, sh, ws=ws[1])
+        eager = gsc.gsc_plan_reorder(ctx, pos, sh, ws=ws[0], stream=other)
+    other.synchronize()
+    graph.replay()
+    torch.cuda.synchronize()
+    for k in range(2):
+        assert torch.equal(got[k], want[k])
+    del eager
