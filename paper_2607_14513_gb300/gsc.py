@@ -260,8 +260,10 @@ def _addr(t):
 
 def _stream(stream):
     import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return C.c_void_p(stream.cuda_stream)
+    # the current stream's handle without a Stream object: 0.5 us, against 3.1 us of a call's 17
+    return C.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 class Context:
