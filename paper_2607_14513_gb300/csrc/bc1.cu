@@ -71,10 +71,7 @@ __global__ void __launch_bounds__(32 * BC1_WARPS, 4)
         stage_groups<BPW + 1>(sh, perm, T, (b0 + i) / 16, n_groups,
                               reinterpret_cast<uint32_t(*)[BPW + 1]>(&S[w].tex[0][i]), S[w].raw);
       } else if (b0 + i + lane < total) {
-        const uint8_t* p = texin + (b0 + i + lane) * 48;
-#pragma unroll
-        for (int t = 0; t < 16; t++)
-          S[w].tex[t][i + lane] = (uint32_t)p[3 * t] | ((uint32_t)p[3 * t + 1] << 8) | ((uint32_t)p[3 * t + 2] << 16);
+        stage_texels<BPW + 1>(texin + (b0 + i + lane) * 48, ((uintptr_t)texin & 15) == 0, &S[w].tex[0][i + lane]);
       }
     }
     __syncwarp();

@@ -65,8 +65,9 @@ __device__ __forceinline__ Bc1Res bc1_eval_k(const uint32_t (&tx)[16], int base,
   return r;
 }
 
-// clamp(round_div(num, den), 0, 255), half away from zero, as round_div255 but in 32 bits: |num| < 2^23, 0 < den <
-// 2^15. rcp: 1 / (2 den), rounded.
+// clamp(round_div(num, den), 0, 255), half away from zero, for |num| < 2^23 and 0 < den < 2^15; rcp: 1 / (2 den),
+// rounded. A negative numerator clamps to 0; the float quotient of floor((2 num + den) / (2 den)) is off by at most
+// one, and one exact step each way lands on it.
 __device__ __forceinline__ int bc1_ratio(int num, int den, float rcp) {
   if (num < 0) return 0;
   const int D = 2 * den, N = 2 * num + den;

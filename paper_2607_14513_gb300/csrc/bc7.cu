@@ -210,10 +210,7 @@ __global__ void __launch_bounds__(32 * BC7_WARPS, BC7_MIN_BLOCKS)
                                   reinterpret_cast<uint32_t*>(S[w].r));
       col0 = (int)(b0 - g0 * 16);
     } else if (live) {
-      const uint8_t* p = texin + blk * 48;
-#pragma unroll
-      for (int t = 0; t < 16; t++)
-        S[w].tex[t][lane] = (uint32_t)p[3 * t] | ((uint32_t)p[3 * t + 1] << 8) | ((uint32_t)p[3 * t + 2] << 16);
+      stage_texels<BC7_STRIDE>(texin + blk * 48, ((uintptr_t)texin & 15) == 0, &S[w].tex[0][lane]);
     } else {
 #pragma unroll
       for (int t = 0; t < 16; t++) S[w].tex[t][lane] = 0x808080u;

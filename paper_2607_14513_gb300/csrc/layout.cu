@@ -1,50 +1,54 @@
 // layout.cu -- fixed codings of any block layout (Sec. IV-B, Figs. SetupA / SetupB / SetupD;
 // Table I's BC1, BC7 and "BC7 on the first block(s), BC1 on the rest" rows).
 //
-// Three steps on the caller's stream: one thread per slot quantises its Gaussian (Sec. V-A)
-// and scatters the 16 texels to their blocks, BC7 blocks and BC1 blocks into two dense texel
+// Three steps on the caller's stream: the Gaussians are quantised (Sec. V-A) and their 16 texels
+// go to their blocks, BC7 blocks and BC1 blocks into two dense texel
 // arrays in output order; the block encoders code each array (the same search as every other
 // coding); an interleave writes every group's BC7 blocks then its BC1 blocks. A coding with
 // one format writes the encoder's output in place and skips the interleave.
 #include "gsc_internal.cuh"
 #include "layout.cuh"
+#include "stage.cuh"
 
 namespace {
 
-__global__ void k_stage_layout(const float* __restrict__ sh, const int32_t* __restrict__ perm,
+// A warp stages two groups (stage.cuh: coefficient c of slot u at tile[u][c]); a lane then collects one block's texels
+// and stores its 48 bytes in 16-byte pieces. 300,000 Gaussians in
+// layout B: 18 us, the whole call 518 us, against 563 us with a slot per thread that read a row alone and stored bytes.
+#define LAY_WARPS 4
+__global__ void __launch_bounds__(32 * LAY_WARPS) k_stage_layout(const float* __restrict__ sh, const int32_t* __restrict__ perm,
                                const float* __restrict__ scales, int64_t n_groups, int layout, int j,
                                uint8_t* __restrict__ tex7, uint8_t* __restrict__ tex1) {
-  __shared__ float s_scale[16];
-  if (threadIdx.x < 16) s_scale[threadIdx.x] = scales[threadIdx.x];
+  __shared__ StageScale T;
+  __shared__ uint32_t tile[LAY_WARPS][16][33];
+  __shared__ uint32_t raw[LAY_WARPS][STAGE_RAW];
+  if (threadIdx.x < 32) stage_scales(T, scales);
   __syncthreads();
-  const int64_t ns = n_groups * 16;
-  for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < ns; s += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t g = s >> 4;
-    const int u = (int)(s & 15);
-    // a padding slot repeats the last valid slot before it in its group (none: texel 128)
-    int32_t src = __ldg(perm + s);
-    for (int v = u - 1; src < 0 && v >= 0; v--) src = __ldg(perm + g * 16 + v);
-    float x[48];
-    if (src >= 0) {
-      const float4* p = reinterpret_cast<const float4*>(sh + (int64_t)src * 48);
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, k = lane & 15;
+  const bool b7 = lay_bc7(layout, j, k);
+  const int r = lay_rank(layout, j, k);
+  for (int64_t g0 = ((int64_t)blockIdx.x * LAY_WARPS + w) * 2; g0 < n_groups; g0 += (int64_t)gridDim.x * LAY_WARPS * 2) {
+    stage_groups<33>(sh, perm, T, g0, n_groups, tile[w], raw[w]);
+    const int64_t g = g0 + (lane >> 4);
+    if (g < n_groups) {
+      uint32_t x[16], v[12];
 #pragma unroll
-      for (int i = 0; i < 12; i++) {
-        const float4 f = __ldg(p + i);
-        x[4 * i] = f.x; x[4 * i + 1] = f.y; x[4 * i + 2] = f.z; x[4 * i + 3] = f.w;
+      for (int t = 0; t < 16; t++) {
+        int u, c;
+        lay_at(layout, k, t, u, c);
+        x[t] = tile[w][u][(lane & 16) + c];
       }
-    }
 #pragma unroll
-    for (int c = 0; c < 16; c++) {
-      int k, t;
-      lay_inv(layout, u, c, k, t);
-      const bool b7 = lay_bc7(layout, j, k);
-      const int r = lay_rank(layout, j, k);
-      uint8_t* d = b7 ? tex7 + ((g * j + r) * 16 + t) * 3 : tex1 + ((g * (16 - j) + r) * 16 + t) * 3;
-      const float sk = s_scale[c];
-      d[0] = src >= 0 ? (uint8_t)gsc_quant1(x[3 * c], sk) : 128;
-      d[1] = src >= 0 ? (uint8_t)gsc_quant1(x[3 * c + 1], sk) : 128;
-      d[2] = src >= 0 ? (uint8_t)gsc_quant1(x[3 * c + 2], sk) : 128;
+      for (int q = 0; q < 4; q++) {
+        v[3 * q] = __byte_perm(x[4 * q], x[4 * q + 1], 0x4210);
+        v[3 * q + 1] = __byte_perm(x[4 * q + 1], x[4 * q + 2], 0x5421);
+        v[3 * q + 2] = __byte_perm(x[4 * q + 2], x[4 * q + 3], 0x6542);
+      }
+      uint4* d = reinterpret_cast<uint4*>(b7 ? tex7 + (g * j + r) * 48 : tex1 + (g * (16 - j) + r) * 48);
+#pragma unroll
+      for (int q = 0; q < 3; q++) d[q] = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
     }
+    __syncwarp();
   }
 }
 
@@ -103,7 +107,7 @@ gsc_status layout_encode_run(gsc_ctx* c, const float* sh, int64_t n, const int32
   const LayoutWs L = carve_layout(ws, ws_bytes, ng, j, &ok);
   if (!ws || !ok) return GSC_ERR_OOM;
   gsc_count_launch();
-  k_stage_layout<<<grid_of(ng * 16), 256, 0, st>>>(sh, perm, scales, ng, layout, j, L.tex7, L.tex1);
+  k_stage_layout<<<grid_of(ng * 16), 32 * LAY_WARPS, 0, st>>>(sh, perm, scales, ng, layout, j, L.tex7, L.tex1);
   GSC_CUDA(cudaGetLastError());
   if (j > 0) {
     GscTimed tm(c, T_BC7, st);

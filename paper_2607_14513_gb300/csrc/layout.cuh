@@ -18,6 +18,13 @@ __host__ __device__ __forceinline__ void lay_inv(int layout, int u, int c, int& 
   else { k = c; t = u; }
 }
 
+// block k, texel t -> slot u, coefficient c
+__host__ __device__ __forceinline__ void lay_at(int layout, int k, int t, int& u, int& c) {
+  if (layout == GSC_LAYOUT_A) { u = k; c = t; }
+  else if (layout == GSC_LAYOUT_B) { u = (k & ~3) | (t >> 2); c = ((k & 3) << 2) | (t & 3); }
+  else { u = t; c = k; }
+}
+
 __host__ __device__ __forceinline__ bool lay_bc7(int layout, int j, int k) {
   if (layout == GSC_LAYOUT_A) return j == 16;
   if (layout == GSC_LAYOUT_B) return (k & 3) < (j >> 2);

@@ -52,6 +52,15 @@ __device__ __forceinline__ uint32_t stage_quant4(float4 x, float4 s, float4 r) {
   return __byte_perm(lo, hi, 0x5410);
 }
 
+// Four texels of three bytes from three words, STEP words apart.
+template <int STEP>
+__device__ __forceinline__ void stage_unpack(uint32_t a, uint32_t b, uint32_t c, uint32_t* to) {
+  to[0] = a & 0xFFFFFFu;
+  to[STEP] = __funnelshift_r(a, b, 24) & 0xFFFFFFu;
+  to[2 * STEP] = __funnelshift_r(b, c, 16) & 0xFFFFFFu;
+  to[3 * STEP] = c >> 8;
+}
+
 // By one warp: groups g0 and g0 + 1 (those below n_groups) into the 32 columns of tex. STRIDE: words between texel
 // rows, one more than a multiple of 32. raw: STAGE_RAW words. STEPS: eighths of rows read ahead, times 8 rows
 // (4: all in flight together; 1: a quarter of the code).
@@ -101,46 +110,25 @@ __device__ __forceinline__ void stage_groups(const float* __restrict__ sh, const
   }
   __syncwarp();
   const uint32_t* q = raw + lane * 13;
-  const int col = lane & 16;
 #pragma unroll
-  for (int j = 0; j < 4; j++) {
-    const uint32_t a = q[3 * j], b = q[3 * j + 1], c = q[3 * j + 2];
-    tex[t][col + 4 * j] = a & 0xFFFFFFu;
-    tex[t][col + 4 * j + 1] = __funnelshift_r(a, b, 24) & 0xFFFFFFu;
-    tex[t][col + 4 * j + 2] = __funnelshift_r(b, c, 16) & 0xFFFFFFu;
-    tex[t][col + 4 * j + 3] = c >> 8;
-  }
+  for (int j = 0; j < 4; j++) stage_unpack<1>(q[3 * j], q[3 * j + 1], q[3 * j + 2], &tex[t][(lane & 16) + 4 * j]);
   __syncwarp();
 }
 
-__device__ __forceinline__ int tex_r(uint32_t v) { return v & 255; }
-__device__ __forceinline__ int tex_g(uint32_t v) { return (v >> 8) & 255; }
-__device__ __forceinline__ int tex_b(uint32_t v) { return (v >> 16) & 255; }
-
-// Exact clamp(round_div(num, den), 0, 255) for den > 0, round_div rounding half away from zero,
-// for several numerators over one denominator: a negative numerator clamps to 0; otherwise
-// floor((2num + den) / (2den)) is estimated in float with one reciprocal of 2den per
-// denominator and corrected exactly in 64-bit integers. The quotient is below 256 and the
-// conversions, the reciprocal and the product carry a relative error of a few 2^-24, so the
-// estimate's floor is off by at most one and one exact step each way lands on it.
-struct RoundDiv255 {
-  long long D;  // 2 den
-  float rcp;    // 1 / D, rounded
-};
-__device__ __forceinline__ RoundDiv255 round_div255_of(long long den) {
-  RoundDiv255 r;
-  r.D = 2 * den;
-  r.rcp = __frcp_rn((float)r.D);
-  return r;
+// A block's 48 bytes of texels into column `col` of a tile (its first row's word; STRIDE words between rows). wide: the
+// array starts on a 16-byte boundary.
+template <int STRIDE>
+__device__ __forceinline__ void stage_texels(const uint8_t* __restrict__ p, bool wide, uint32_t* col) {
+  if (wide) {
+    const uint4* q = reinterpret_cast<const uint4*>(p);
+    const uint4 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
+    stage_unpack<STRIDE>(a.x, a.y, a.z, col);
+    stage_unpack<STRIDE>(a.w, b.x, b.y, col + 4 * STRIDE);
+    stage_unpack<STRIDE>(b.z, b.w, c.x, col + 8 * STRIDE);
+    stage_unpack<STRIDE>(c.y, c.z, c.w, col + 12 * STRIDE);
+  } else {
+#pragma unroll 1
+    for (int t = 0; t < 16; t++)
+      col[t * STRIDE] = (uint32_t)p[3 * t] | ((uint32_t)p[3 * t + 1] << 8) | ((uint32_t)p[3 * t + 2] << 16);
+  }
 }
-__device__ __forceinline__ int round_div255(const RoundDiv255& r, long long num) {
-  if (num < 0) return 0;
-  const long long N = 2 * num + r.D / 2;
-  if (N >= 256 * r.D) return 255;
-  int q = (int)((float)N * r.rcp);
-  q = min(max(q, 0), 255);
-  if (q > 0 && (long long)q * r.D > N) q--;
-  if (q < 255 && (long long)(q + 1) * r.D <= N) q++;
-  return q;
-}
-
