@@ -43,20 +43,17 @@ RATE_TARGET_X4 = 24          # 6 bits per coefficient texel
 N_CAMS = 8
 # BC7 search: palette-distance evaluations per block (the candidate enumeration of the
 # encoder: initial indices + every p-bit combination, per mode / partition / rotation /
-# index selection), and integer operations per evaluation (3 differences, 3 squares
-# accumulated, compare, select).
+# index selection). The search finds the least error over all of it but leaves out, exactly,
+# the candidates that a bound shows to be worse, so this counts the result's cost, not the kernel's.
 BC7_EVALS_PER_BLOCK = (16 * (16 * 8 + 4 * 16 * 8) + 64 * (16 * 8 + 2 * 16 * 8) + 64 * (16 * 4 + 16 * 4)
                        + 64 * (16 * 4 + 4 * 16 * 4) + (128 + 256 + 3 * 768) + (128 + 3 * 256)
                        + (16 * 16 + 4 * 16 * 16) + 64 * (16 * 4 + 4 * 16 * 4))
-# integer operations of one palette evaluation as the search kernel computes it (best_key in
-# csrc/bc7.cu): the byte dot product of texel and entry, the entry's key minus 32 x that product,
-# and the running minimum; gsc_probe_op_rate kind 5 runs exactly this mix
-OPS_PER_EVAL = 3
 # per launch, measured with ncu for the kernels as they stand (to be reset to None when a kernel
 # changes): DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) on the 3M-Gaussian workload,
-# and the BC7 search's thread instructions per block (smsp__thread_inst_executed.sum / blocks)
-MEASURED_TRAFFIC = {"scene3m": {"k_bc7": None, "k_eval2_bc7_slots": 324060000, "k_eval_tex_bc7": 388227328}}
-MEASURED_BC7_THREAD_INSTR_PER_BLOCK = 582878   # 262,144-Gaussian scene (the search is exhaustive: size-independent)
+# and the BC7 search's thread instructions per block (smsp__thread_inst_executed.sum / blocks), which
+# depend on the data
+MEASURED_TRAFFIC = {"scene3m": {"k_bc7": None, "k_eval2_bc7_slots": 324180000, "k_eval_tex_bc7": 388227328}}
+MEASURED_BC7_THREAD_INSTR_PER_BLOCK = {"scene3m": 234686}
 ISSUE_LANES_PER_CLK_SM = 128   # 4 schedulers x 32 lanes, one warp instruction each per clock
 
 
@@ -255,8 +252,9 @@ def run_gsc(args, world, rank, local):
     # dominant kernel: the BC7 search (integer ALU bound)
     bc7_ms = kt["bc7_encode"][0] / max(1, kt["bc7_encode"][1])
     roofline = bc7_roofline(ctx, gsc, stream, dev, clk, BC7_EVALS_PER_BLOCK * ns, bc7_ms,
-                            "k_bc7 (BC7 candidate search, thread per block)", ns,
-                            MEASURED_TRAFFIC.get(args.workload, {}).get("k_bc7"))
+                            "k_bc7 (BC7 candidate search, a warp per 32 blocks)", ns,
+                            MEASURED_TRAFFIC.get(args.workload, {}).get("k_bc7"),
+                            MEASURED_BC7_THREAD_INSTR_PER_BLOCK.get(args.workload))
     # the fused decode + SH evaluation (HBM bound) of each coding, timed alone after the step, with
     # the centres resident in slot order (the step's own gsc_positions_to_slots output): algorithmic
     # bytes per launch = the coded blocks + 4 B slot entry + 12 B centre + 8 x 12 B output per Gaussian
@@ -355,34 +353,27 @@ def run_gsc(args, world, rank, local):
     return out
 
 
-def bc7_roofline(ctx, gsc, stream, dev, clk, evals, ms, kernel, blocks, traffic):
-    """The BC7 search against the measured rate of its own evaluation mix (gsc_probe_op_rate kind 5),
-    and against the SM's issue ceiling (128 lanes per clock per SM at the sampled SM clock), with the
-    per-instruction probe rates beside them."""
+def bc7_roofline(ctx, gsc, stream, dev, clk, evals, ms, kernel, blocks, traffic, instr=None):
+    """The BC7 search against the SM's issue ceiling (128 lanes per clock per SM at the sampled SM
+    clock), in thread instructions as counted on this workload (instr per block; None where they were
+    not counted). The enumeration's evaluations per second and the probe rates stand beside it."""
     import torch
     probes = {gsc.PROBE_KINDS[k]: gsc.op_rate(ctx, k, stream=stream) for k in sorted(gsc.PROBE_KINDS)}
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     mhz = clk.get("sm_mhz") or 2070.0
     per_clk = {k: round(v / (sms * mhz * 1e6), 2) for k, v in probes.items()}
     issue = sms * ISSUE_LANES_PER_CLK_SM * mhz * 1e6
-    peak = probes["bc7_palette_eval"]
-    ops = evals * OPS_PER_EVAL
-    ach = ops / (ms * 1e-3)
-    out = {"bound": "alu", "achieved": round(ach / 1e12, 3), "peak": round(peak / 1e12, 3), "unit": "Tops/s",
-           "frac": round(ach / peak, 4), "traffic": traffic, "kernel": kernel,
-           "peak_source": "measured on this GPU: gsc_probe_op_rate kind 5, the evaluation's own mix (dp4a, "
-                          "scaled key, minimum) in independent chains at full occupancy",
-           "algorithmic": "%d palette evaluations x %d int ops (dot, key, minimum), %d blocks"
-                          % (evals // max(1, blocks), OPS_PER_EVAL, blocks),
-           "issue_ceiling_Tops_s": round(issue / 1e12, 3), "frac_of_issue_ceiling": round(ach / issue, 4),
-           "probes_Tops_s": {k: round(v / 1e12, 3) for k, v in probes.items()},
-           "probes_ops_per_clk_per_sm": per_clk}
-    if MEASURED_BC7_THREAD_INSTR_PER_BLOCK:
-        ti = MEASURED_BC7_THREAD_INSTR_PER_BLOCK * blocks / (ms * 1e-3)
-        out["instructions"] = {"thread_instr_per_block": MEASURED_BC7_THREAD_INSTR_PER_BLOCK,
-                               "thread_instr_per_eval": round(MEASURED_BC7_THREAD_INSTR_PER_BLOCK * blocks / evals, 2),
-                               "Tinstr_s": round(ti / 1e12, 3), "frac_of_issue_ceiling": round(ti / issue, 4)}
-    return out
+    ach = instr * blocks / (ms * 1e-3) if instr else None
+    return {"bound": "instruction issue", "achieved": round(ach / 1e12, 3) if ach else None,
+            "peak": round(issue / 1e12, 3), "unit": "Tinstr/s", "frac": round(ach / issue, 4) if ach else None,
+            "traffic": traffic, "kernel": kernel,
+            "peak_source": "152 SMs x 128 lanes x the sampled SM clock" if sms == 152 else "SMs x 128 lanes x the SM clock",
+            "algorithmic": "least error over %d palette evaluations per block, %d blocks; most are left out by an exact "
+                           "bound" % (evals // max(1, blocks), blocks),
+            "thread_instr_per_block": instr, "Mblocks_s": round(blocks / ms / 1e3, 2),
+            "enumerated_Tevals_s": round(evals / (ms * 1e-3) / 1e12, 3),
+            "probes_Tops_s": {k: round(v / 1e12, 3) for k, v in probes.items()},
+            "probes_ops_per_clk_per_sm": per_clk}
 
 
 def time_bc7_mappings(ctx, gsc, stream, sh, perm, scales, n):
