@@ -294,6 +294,7 @@ gsc_status ctx_new(int device, bool init_tables, gsc_ctx** out) {
     if (e == cudaSuccess) e = bc1_init_tables();
     if (e == cudaSuccess) e = bc7_init_tables();
     if (e == cudaSuccess) e = decode_init_tables();
+    if (e == cudaSuccess) e = bc7_init_kernels();
     if (e == cudaSuccess) e = plan_init();
     if (e == cudaSuccess) e = cudaDeviceSynchronize();
   }

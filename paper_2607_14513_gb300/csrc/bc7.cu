@@ -149,22 +149,27 @@ cudaError_t bc7_init_tables() {
 }
 
 // One kernel for both sources: staged layout-D groups (sh / perm / scales) or raw
-// texels [nblk][16][3] (texin != nullptr), so the search is compiled once. A CTA is four warps that
-// share the quantisation tables and nothing else: each warp stages its own 32 blocks (two groups) and
-// searches them at its own pace. Bound by instruction issue and fetch (64% of the issue slots; a quarter of the
-// stalls are fetch). 5 CTAs (20 warps, at most 102 registers) per SM: 320,000 blocks of the scene with outliers
-// 3.85 ms, against 3.92 ms with 6 CTAs (80 registers) and 4.03 ms with 4. 3M blocks of that scene: 36.9 ms, against
-// 67.0 ms for the exhaustive search; 262,144 without outliers: 1.37 against 6.95 ms.
+// texels [nblk][16][3] (texin != nullptr), so the search is compiled once. The warps of a CTA share the
+// quantisation tables, each stages and searches its own 32 blocks (two groups), and they go from phase to phase
+// together: bound by instruction issue and fetch, and warps in one phase run the same code. With barriers between the
+// phases and before the solve, and ten warps per CTA, 3M blocks of the scene with outliers take 28.7 ms, against 34.5 ms
+// with each of four warps at its own pace and 67.0 ms for the exhaustive search; 262,144 without outliers: 1.21, 1.39
+// and 6.95 ms. 20 warps per SM at most 102 registers; 24 at 80 and 16 at 128 were slower.
 #define BC7_WARPS 4
 // Up to this many blocks per SM a warp takes 8 blocks instead of 32: the chip has warps to spare and the time is
-// one warp's. Scene without outliers, 8 against 32 blocks per warp: 4,096 blocks 187 against 265 us, 10,000 209
-// against 268 us, 20,000 294 against 291 us, 40,000 521 against 335 us.
+// one warp's. Scene without outliers, 8 against 32 blocks per warp, each at its own pace: 4,096 blocks 187 against 265 us,
+// 10,000 209 against 268 us, 20,000 294 against 291 us, 40,000 521 against 335 us.
 #define BC7_FEW 112
 #define BC7_MIN_BLOCKS 5
+// Above this many blocks per SM a CTA has ten warps instead of four: more warps share their phase's code, but a CTA of
+// 320 blocks leaves a larger part of the last wave idle. Ten against four: 120,000 blocks 694 against 673 us, 262,144
+// 1252 against 1279 us, the scene of 3M 31.1 against 34.3 ms; twenty: 120,000 801, 262,144 1200 us, 3M 31.2 ms.
+#define BC7_MANY 1280
+#define BC7_WIDE 10
 
 // the warp's staged blocks (columns col0.. of its tile): search, solve, store. blk: this lane's block, live:
 // whether it exists (lanes from BPW on have none)
-template <int BPW>
+template <int BPW, bool SYNC>
 __device__ __forceinline__ void bc7_finish(Bc7Warp& W, int col0, bool live, int64_t blk, const uint8_t* sq,
                                            uint4* __restrict__ blocks, uint32_t* __restrict__ sse7,
                                            uint64_t* __restrict__ sse64) {
@@ -172,7 +177,8 @@ __device__ __forceinline__ void bc7_finish(Bc7Warp& W, int col0, bool live, int6
   const uint32_t* my = &W.tex[0][col0 + lane % BPW];
   uint4 out;
   const bool constant = const_block(my, &out);
-  bc7_search<BPW>(W, col0, live && !constant, sq);
+  bc7_search<BPW, SYNC>(W, col0, live && !constant, sq);
+  if (SYNC) __syncthreads();
   if (live) {
     uint32_t err = 0;
     if (!constant) {
@@ -186,12 +192,13 @@ __device__ __forceinline__ void bc7_finish(Bc7Warp& W, int col0, bool live, int6
   }
 }
 
-template <int BPW>
-__global__ void __launch_bounds__(32 * BC7_WARPS, BC7_MIN_BLOCKS)
+template <int BPW, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 20 / WARPS)
     k_bc7(const float* __restrict__ sh, const int32_t* __restrict__ perm, const float* __restrict__ scales,
           int64_t n_groups, const uint8_t* __restrict__ texin, int64_t nblk, uint4* __restrict__ blocks,
           uint32_t* __restrict__ sse7, uint64_t* __restrict__ sse64) {
-  __shared__ Bc7Warp S[BC7_WARPS];
+  extern __shared__ __align__(16) uint8_t dyn[];
+  Bc7Warp* S = reinterpret_cast<Bc7Warp*>(dyn);
   __shared__ StageScale T;
   __shared__ uint8_t sq[12 * 256];
   for (int i = threadIdx.x; i < 12 * 256; i += blockDim.x) sq[i] = (&g_qtab[0][0])[i];
@@ -199,14 +206,16 @@ __global__ void __launch_bounds__(32 * BC7_WARPS, BC7_MIN_BLOCKS)
   __syncthreads();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t total = texin ? nblk : n_groups * 16;
-  for (int64_t b0 = ((int64_t)blockIdx.x * BC7_WARPS + w) * BPW; b0 < total; b0 += (int64_t)gridDim.x * BC7_WARPS * BPW) {
+  // every warp of the CTA goes through the phases, one without blocks too
+  for (int64_t c0 = (int64_t)blockIdx.x * WARPS * BPW; c0 < total; c0 += (int64_t)gridDim.x * WARPS * BPW) {
+    const int64_t b0 = c0 + w * BPW;
     const int64_t blk = b0 + lane;
     const bool live = lane < BPW && blk < total;
     int col0 = 0;
     if (!texin) {
       // two groups, or the one that holds the warp's eight blocks
       const int64_t g0 = b0 / 16;
-      stage_groups<BC7_STRIDE, 1>(sh, perm, T, g0, BPW == 32 ? n_groups : g0 + 1, S[w].tex,
+      stage_groups<BC7_STRIDE, 1>(sh, perm, T, g0, BPW == 32 ? n_groups : min(g0 + 1, n_groups), S[w].tex,
                                   reinterpret_cast<uint32_t*>(S[w].r));
       col0 = (int)(b0 - g0 * 16);
     } else if (live) {
@@ -216,7 +225,7 @@ __global__ void __launch_bounds__(32 * BC7_WARPS, BC7_MIN_BLOCKS)
       for (int t = 0; t < 16; t++) S[w].tex[t][lane] = 0x808080u;
     }
     __syncwarp();
-    bc7_finish<BPW>(S[w], col0, live, blk, sq, blocks, sse7, sse64);
+    bc7_finish<BPW, true>(S[w], col0, live, blk, sq, blocks, sse7, sse64);
     __syncwarp();
   }
 }
@@ -225,16 +234,23 @@ static cudaError_t launch_bc7(const float* sh, const int32_t* perm, const float*
                               const uint8_t* tex, int64_t nblk, uint8_t* out, uint32_t* sse7, uint64_t* sse64,
                               cudaStream_t st) {
   const int64_t total = tex ? nblk : n_groups * 16;
-  const bool few = total <= (int64_t)gsc_sm_count() * BC7_FEW;
-  const int64_t grid = std::min<int64_t>(ceil_div64(total, (few ? 8 : 32) * BC7_WARPS), 0x7FFFFFFF);
+  const bool few = total <= (int64_t)gsc_sm_count() * BC7_FEW, many = total > (int64_t)gsc_sm_count() * BC7_MANY;
+  const int warps = many ? BC7_WIDE : BC7_WARPS;
+  const int64_t grid = std::min<int64_t>(ceil_div64(total, (few ? 8 : 32) * warps), 0x7FFFFFFF);
+  const size_t smem = warps * sizeof(Bc7Warp);
+  uint4* to = reinterpret_cast<uint4*>(out);
   gsc_count_launch();
-  if (few)
-    k_bc7<8><<<(int)grid, 32 * BC7_WARPS, 0, st>>>(sh, perm, scales, n_groups, tex, nblk, reinterpret_cast<uint4*>(out),
-                                                   sse7, sse64);
-  else
-    k_bc7<32><<<(int)grid, 32 * BC7_WARPS, 0, st>>>(sh, perm, scales, n_groups, tex, nblk,
-                                                    reinterpret_cast<uint4*>(out), sse7, sse64);
+  if (few) k_bc7<8, BC7_WARPS><<<(int)grid, 32 * warps, smem, st>>>(sh, perm, scales, n_groups, tex, nblk, to, sse7, sse64);
+  else if (many) k_bc7<32, BC7_WIDE><<<(int)grid, 32 * warps, smem, st>>>(sh, perm, scales, n_groups, tex, nblk, to, sse7, sse64);
+  else k_bc7<32, BC7_WARPS><<<(int)grid, 32 * warps, smem, st>>>(sh, perm, scales, n_groups, tex, nblk, to, sse7, sse64);
   return cudaGetLastError();
+}
+
+cudaError_t bc7_init_kernels() {  // dynamic shared memory above 48 KB, once per device
+  cudaError_t e = cudaFuncSetAttribute(k_bc7<32, BC7_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)(BC7_WIDE * sizeof(Bc7Warp)));
+  return e == cudaSuccess ? cudaFuncSetAttribute(k_bc7<8, BC7_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)(BC7_WARPS * sizeof(Bc7Warp))) : e;
 }
 
 cudaError_t launch_bc7_groups(const float* sh, const int32_t* perm, const float* scales, int64_t n_groups,
@@ -315,7 +331,7 @@ __global__ void __launch_bounds__(32 * BC7_WARPS, BC7_MIN_BLOCKS)
       stage_groups<BC7_STRIDE, 1>(S.sh, S.perm, T[w], g0, S.n_groups, W[w].tex, reinterpret_cast<uint32_t*>(W[w].r));
       const int64_t blk = g0 * 16 + lane;
       const bool live = g0 + (lane >> 4) < gend;
-      bc7_finish<32>(W[w], 0, live, blk, sq, reinterpret_cast<uint4*>(S.b7), S.sse7, nullptr);
+      bc7_finish<32, false>(W[w], 0, live, blk, sq, reinterpret_cast<uint4*>(S.b7), S.sse7, nullptr);
       __syncwarp();
     }
   }

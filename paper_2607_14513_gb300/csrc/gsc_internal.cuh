@@ -136,6 +136,7 @@ cudaError_t launch_bc1_blocks(const uint8_t* tex, int64_t nblk, uint8_t* out, ui
 
 // bc7.cu
 cudaError_t bc7_init_tables();
+cudaError_t bc7_init_kernels();
 cudaError_t launch_bc7_groups(const float* sh, const int32_t* perm, const float* scales, int64_t n_groups,
                               uint8_t* blocks, uint32_t* sse7, cudaStream_t st);
 cudaError_t launch_bc7_blocks(const uint8_t* tex, int64_t nblk, uint8_t* out, uint64_t* sse, cudaStream_t st);

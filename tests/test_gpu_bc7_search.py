@@ -53,3 +53,19 @@ def test_pruned_search_is_the_exhaustive_one(ctx, O, kind, n):
     torch.cuda.synchronize()
     assert np.array_equal(gsse.cpu().numpy().astype(np.uint64), osse)
     assert np.array_equal(gb.cpu().numpy(), ob)
+
+
+@pytest.mark.parametrize("n", [20_001, 200_003])
+def test_pruned_search_in_wider_launches(ctx, O, n):
+    """A warp per 32 blocks, in CTAs of four warps and (beyond 1280 blocks per SM) of ten, the last CTA partly empty:
+    repeated blocks of every kind, against the oracle's coding of each."""
+    from paper_2607_14513_gb300 import gsc
+    rng = np.random.default_rng(n)
+    kinds = ["ramp", "near", "line", "noise", "outliers", "extreme", "ties"]
+    tex = np.clip(np.concatenate([_content(k, 101, rng) for k in kinds]), 0, 255).astype(np.uint8)
+    ob, osse = O.encode_blocks(tex, 7)
+    at = rng.integers(0, tex.shape[0], size=n)
+    gb, gsse = gsc.gsc_encode_blocks(ctx, torch.from_numpy(tex[at]).cuda(), gsc.FMT_BC7)
+    torch.cuda.synchronize()
+    assert np.array_equal(gsse.cpu().numpy().astype(np.uint64), osse[at])
+    assert np.array_equal(gb.cpu().numpy(), ob[at])
