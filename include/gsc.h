@@ -363,8 +363,9 @@ typedef struct {
 
 /* How the encode launch hands out work: schedule 0 = static round robin over tiles, 1 = atomic
  * work queue, 2 = atomic queue, 3 = one CTA unit per tile; schedules other than 1 list the scenes
- * by decreasing cost. CTAs per SM 1..32 (schedules 0-2; a CTA is four warps that claim their own tiles; 4
- * BC1 CTAs fit per SM; for BC7 the number counts fives of CTAs, one five fits per SM; above what fits the grid is oversubscribed and the hardware block scheduler balances);
+ * by decreasing cost. CTAs per SM 1..32 (schedules 0-2; a BC1 CTA is four warps that claim their own
+ * tiles, 4 CTAs fit per SM; a BC7 CTA claims a tile for its four warps, and the number counts fives of CTAs,
+ * one five fits per SM; above what fits the grid is oversubscribed and the hardware block scheduler balances);
  * groups per BC1 tile (multiple of 8; BC7 tiles are 8 groups). The plans of the scenes run on 4 streams at once. */
 typedef struct {
   int32_t schedule;

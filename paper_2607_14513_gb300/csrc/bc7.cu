@@ -169,7 +169,7 @@ cudaError_t bc7_init_tables() {
 
 // the warp's staged blocks (columns col0.. of its tile): search, solve, store. blk: this lane's block, live:
 // whether it exists (lanes from BPW on have none)
-template <int BPW, bool SYNC>
+template <int BPW>
 __device__ __forceinline__ void bc7_finish(Bc7Warp& W, int col0, bool live, int64_t blk, const uint8_t* sq,
                                            uint4* __restrict__ blocks, uint32_t* __restrict__ sse7,
                                            uint64_t* __restrict__ sse64) {
@@ -177,8 +177,8 @@ __device__ __forceinline__ void bc7_finish(Bc7Warp& W, int col0, bool live, int6
   const uint32_t* my = &W.tex[0][col0 + lane % BPW];
   uint4 out;
   const bool constant = const_block(my, &out);
-  bc7_search<BPW, SYNC>(W, col0, live && !constant, sq);
-  if (SYNC) __syncthreads();
+  bc7_search<BPW>(W, col0, live && !constant, sq);
+  __syncthreads();
   if (live) {
     uint32_t err = 0;
     if (!constant) {
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(32 * WARPS, 20 / WARPS)
       for (int t = 0; t < 16; t++) S[w].tex[t][lane] = 0x808080u;
     }
     __syncwarp();
-    bc7_finish<BPW, true>(S[w], col0, live, blk, sq, blocks, sse7, sse64);
+    bc7_finish<BPW>(S[w], col0, live, blk, sq, blocks, sse7, sse64);
     __syncwarp();
   }
 }
@@ -267,8 +267,8 @@ cudaError_t launch_bc7_blocks(const uint8_t* tex, int64_t nblk, uint8_t* out, ui
 // ---- persistent multi-scene encode -----------------------------------------------------------
 // One launch per coding over the tiles of every listed scene. Tiles
 // are claimed round robin (schedule 0), from an atomic work queue (1, 2), or one per claiming unit
-// (3, a grid of all tiles); a tile finds its scene by binary search over the list. The four warps of a CTA claim
-// their own tiles and walk them 8 groups (BC1) or two (BC7) at a time, since their searches differ in length. The
+// (3, a grid of all tiles); a tile finds its scene by binary search over the list. A BC1 CTA's four
+// warps claim their own tiles and walk them 8 groups at a time, a BC7 CTA claims one for its four warps. The
 // bits equal the single-scene kernels'.
 __device__ __forceinline__ int64_t claim_tile(int schedule, int64_t it, int w, int lane, int* counter) {
   long long ti = 0;
@@ -311,27 +311,32 @@ __global__ void __launch_bounds__(32 * BC7_WARPS, 4)
   }
 }
 
+// The CTA claims a tile for its four warps, which take two groups each and search in step (as in k_bc7).
 __global__ void __launch_bounds__(32 * BC7_WARPS, BC7_MIN_BLOCKS)
     k_batch7(const BatchSceneDev* __restrict__ scenes, int n_scenes, int64_t n_tiles, int schedule,
              int* __restrict__ counter) {
   __shared__ Bc7Warp W[BC7_WARPS];
   __shared__ StageScale T[BC7_WARPS];
+  __shared__ long long s_tile;
   __shared__ uint8_t sq[12 * 256];
   for (int i = threadIdx.x; i < 12 * 256; i += blockDim.x) sq[i] = (&g_qtab[0][0])[i];
-  __syncthreads();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int64_t it = 0;; it++) {
-    const int64_t ti = claim_tile(schedule, it, w, lane, counter);
+    __syncthreads();  // the last tile's number has been read
+    if (threadIdx.x == 0)
+      s_tile = (schedule == 0 || schedule == 3) ? (long long)(blockIdx.x + it * gridDim.x) : (long long)atomicAdd(counter, 1);
+    __syncthreads();
+    const int64_t ti = s_tile;
     if (ti >= n_tiles) break;
     const BatchSceneDev S = scene_of(scenes, n_scenes, ti);
     const int64_t gbeg = (ti - S.tile0) * S.tile_groups, gend = min(gbeg + (int64_t)S.tile_groups, S.work_groups);
     stage_scales(T[w], S.scales);
     __syncwarp();
-    for (int64_t g0 = gbeg; g0 < gend; g0 += 2) {
+    for (int64_t c0 = gbeg; c0 < gend; c0 += 2 * BC7_WARPS) {
+      const int64_t g0 = c0 + 2 * w;
       stage_groups<BC7_STRIDE, 1>(S.sh, S.perm, T[w], g0, S.n_groups, W[w].tex, reinterpret_cast<uint32_t*>(W[w].r));
-      const int64_t blk = g0 * 16 + lane;
       const bool live = g0 + (lane >> 4) < gend;
-      bc7_finish<32, false>(W[w], 0, live, blk, sq, reinterpret_cast<uint4*>(S.b7), S.sse7, nullptr);
+      bc7_finish<32>(W[w], 0, live, g0 * 16 + lane, sq, reinterpret_cast<uint4*>(S.b7), S.sse7, nullptr);
       __syncwarp();
     }
   }
@@ -340,9 +345,9 @@ __global__ void __launch_bounds__(32 * BC7_WARPS, BC7_MIN_BLOCKS)
 cudaError_t launch_batch_encode(int kind, const BatchSceneDev* scenes, int n_scenes, int64_t n_tiles, int schedule,
                                 int ctas_per_sm, int sm_count, int* counter, cudaStream_t st) {
   if (n_tiles <= 0 || n_scenes <= 0) return cudaSuccess;
-  // schedule 3: one claiming unit (a warp) per tile, left to the hardware block scheduler; a BC7 launch has
-  // BC7_MIN_BLOCKS CTAs (what one SM holds) per ctas_per_sm
-  const int64_t cta_tiles = ceil_div64(n_tiles, BC7_WARPS);
+  // schedule 3: one claiming unit (a warp for BC1, a CTA for BC7) per tile, left to the hardware block scheduler; a BC7
+  // launch has BC7_MIN_BLOCKS CTAs (what one SM holds) per ctas_per_sm
+  const int64_t cta_tiles = kind == 7 ? n_tiles : ceil_div64(n_tiles, BC7_WARPS);
   int64_t grid = schedule == 3 ? cta_tiles
                                : (int64_t)(sm_count > 0 ? sm_count : gsc_sm_count()) *
                                      (ctas_per_sm > 0 ? ctas_per_sm : (kind == 7 ? 1 : 4)) *

@@ -458,8 +458,8 @@ __device__ __forceinline__ float bound_unpack(uint16_t h) {
 // Searches the warp's BPW blocks (columns col0.. of its tile; those of the lanes with `active`); leaves each
 // block's least error and its candidate in W.best. All 32 lanes call it. sq: the 12 tables of expanded endpoint
 // values. With fewer than 32 blocks, 32 / BPW lanes share a block's bounds, and the stack serves fewer blocks:
-// the warp is done sooner. SYNC: all warps of the CTA call it, and start each phase together.
-template <int BPW, bool SYNC>
+// the warp is done sooner. All warps of the CTA call it, and start each phase together.
+template <int BPW>
 __device__ __noinline__ void bc7_search(Bc7Warp& W, int col0, bool active, const uint8_t* sq) {
   constexpr int LPB = 32 / BPW;
   const int lane = threadIdx.x & 31, own = lane % BPW, slice = lane / BPW;
@@ -469,7 +469,7 @@ __device__ __noinline__ void bc7_search(Bc7Warp& W, int col0, bool active, const
   int seed = 0;
 #pragma unroll 1
   for (int phase = PH_MODE2; phase <= PH_TWO; phase++) {
-    if (SYNC) __syncthreads();
+    __syncthreads();
     // the phase's bounds, where they are not the last one's (modes 2 and 0 share theirs)
     if (phase == PH_MODE2 || phase == PH_ROT || phase == PH_TWO) {
       const Planes P = planes_of(&W.tex[0][col0 + own]);
