@@ -53,7 +53,7 @@ BC7_EVALS_PER_BLOCK = (16 * (16 * 8 + 4 * 16 * 8) + 64 * (16 * 8 + 2 * 16 * 8) +
 # and the BC7 search's thread instructions per block (smsp__thread_inst_executed.sum / blocks), which
 # depend on the data
 MEASURED_TRAFFIC = {"scene3m": {"k_bc7": None, "k_eval2_bc7_slots": 324180000, "k_eval_tex_bc7": 388227328}}
-MEASURED_BC7_THREAD_INSTR_PER_BLOCK = {"scene3m": 234686}
+MEASURED_BC7_THREAD_INSTR_PER_BLOCK = {"scene3m": 234663}
 ISSUE_LANES_PER_CLK_SM = 128   # 4 schedulers x 32 lanes, one warp instruction each per clock
 
 
