@@ -9,6 +9,7 @@
 // one kernel (decoupled look-back) took 41 us per pass with two resident CTAs per SM and 470 us with four, when
 // most of the machine polled. 32-bit keys where the caller's fit.
 #include "sort.cuh"
+#include "sort_digits.h"
 
 // ---- scan (exclusive, 64-bit) -------------------------------------------------------------
 #define SCAN_BLOCK 1024
@@ -176,10 +177,11 @@ __global__ void __launch_bounds__(256) k_rs_rows(uint32_t* __restrict__ counts, 
   if (t == 0) total[blockIdx.x] = carry;
 }
 
-// vin = nullptr: values are the input positions; kout = nullptr: the sorted keys are not wanted
+// vin = nullptr: values are the input positions; kout = nullptr: the sorted keys are not wanted. mask: the pass's digit
+// as it was counted; BITS, at least as many, is the number of ballots that tell two digits apart.
 template <class K, int BITS>
 __global__ void __launch_bounds__(RS_THREADS, 3)
-    k_rs_scatter(const K* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t n, int shift,
+    k_rs_scatter(const K* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t n, int shift, uint32_t mask,
                  const uint32_t* __restrict__ total, const uint32_t* __restrict__ counts, K* __restrict__ kout,
                  uint32_t* __restrict__ vout) {
   __shared__ K s_key[RS_TILE];
@@ -187,7 +189,6 @@ __global__ void __launch_bounds__(RS_THREADS, 3)
   __shared__ uint32_t s_cnt[RS_WARPS][256];
   __shared__ uint32_t s_start[256], s_base[256];
   __shared__ uint64_t s_scan[8];
-  constexpr uint32_t mask = (1u << BITS) - 1u;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int64_t base = (int64_t)blockIdx.x * RS_TILE;
   const int count = (int)min((int64_t)RS_TILE, n - base);
@@ -236,23 +237,21 @@ __global__ void __launch_bounds__(RS_THREADS, 3)
 template <class K>
 cudaError_t radix_sort(K* keys, K* keys2, uint32_t* vals, uint32_t* vals2, int64_t n, int key_bits, bool iota, bool want_keys,
                        void* state, cudaStream_t st, K** out_keys, uint32_t** out_vals) {
-  const int passes = (key_bits + 7) / 8;
+  const int passes = sort_passes(key_bits);
   uint32_t* total = reinterpret_cast<uint32_t*>(state);
   uint32_t* counts = total + 256;
   const int nt = (int)rs_tiles(n);
-  // the key's bits in equal shares of at most 8
-  for (int p = 0, shift = 0; p < passes && n > 0; p++) {
-    const int bits = (key_bits - shift + passes - p - 1) / (passes - p);
-    gsc_count_launch(); k_rs_count<K><<<nt, RS_THREADS, 0, st>>>(keys, n, shift, (1u << bits) - 1u, counts);
+  for (int p = 0; p < passes && n > 0; p++) {
+    const SortDigit d = sort_digit(key_bits, p);
+    gsc_count_launch(); k_rs_count<K><<<nt, RS_THREADS, 0, st>>>(keys, n, d.shift, d.mask, counts);
     gsc_count_launch(); k_rs_rows<<<256, 256, 0, st>>>(counts, nt, total);
     gsc_count_launch();
     const uint32_t* vin = p == 0 && iota ? nullptr : vals;
     K* kout = p + 1 < passes || want_keys ? keys2 : nullptr;
-    if (bits <= 4) k_rs_scatter<K, 4><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, shift, total, counts, kout, vals2);
-    else if (bits <= 6) k_rs_scatter<K, 6><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, shift, total, counts, kout, vals2);
-    else if (bits == 7) k_rs_scatter<K, 7><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, shift, total, counts, kout, vals2);
-    else k_rs_scatter<K, 8><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, shift, total, counts, kout, vals2);
-    shift += bits;
+    if (d.ballots == 4) k_rs_scatter<K, 4><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, d.shift, d.mask, total, counts, kout, vals2);
+    else if (d.ballots == 6) k_rs_scatter<K, 6><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, d.shift, d.mask, total, counts, kout, vals2);
+    else if (d.ballots == 7) k_rs_scatter<K, 7><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, d.shift, d.mask, total, counts, kout, vals2);
+    else k_rs_scatter<K, 8><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, d.shift, d.mask, total, counts, kout, vals2);
     K* tk = keys; keys = keys2; keys2 = tk;
     uint32_t* tv = vals; vals = vals2; vals2 = tv;
   }
