@@ -225,7 +225,8 @@ __global__ void k_gather_counts(int64_t n, const uint32_t* __restrict__ dval, co
 // One tile key per overlapped tile, emitted in depth order: a stable sort by tile then leaves every
 // tile's list nearest first (equal depths in index order). A warp takes 32 Gaussians and writes their keys
 // together, 32 consecutive ones per step (a thread writing its own Gaussian's keys touched a sector per key:
-// 0.40 ms for the 29M keys of a 1080p frame of 3M Gaussians).
+// 0.40 ms for the 29M keys of a 1080p frame of 3M Gaussians). Steps count from the warp's first key: there are up to
+// 2^32 - 16 keys, and a step past them would wrap.
 template <class K>
 __global__ void __launch_bounds__(256) k_splat_keys(int64_t n, const uint32_t* __restrict__ dval, const int4* __restrict__ rect,
                                                     const uint32_t* __restrict__ count_sorted,
@@ -242,9 +243,11 @@ __global__ void __launch_bounds__(256) k_splat_keys(int64_t n, const uint32_t* _
     const int4 b = c ? rect[i] : make_int4(0, 0, 1, 1);
     const int first = b.y * tiles_x + b.x, wide = b.z - b.x;
     const int last = 31 - __clz(any);
-    const uint32_t begin = __shfl_sync(0xFFFFFFFFu, o, 0), end = __shfl_sync(0xFFFFFFFFu, o + c, last);
-    for (uint32_t e0 = begin; e0 < end; e0 += 32) {
-      const uint32_t e = e0 + lane;
+    const uint32_t begin = __shfl_sync(0xFFFFFFFFu, o, 0), keyed = __shfl_sync(0xFFFFFFFFu, o + c, last) - begin;
+    for (uint32_t k0 = 0; k0 < keyed; k0 += 32) {
+      // past the warp's last key (never written) that key's lane
+      const bool live = k0 + lane < keyed;
+      const uint32_t e = begin + (live ? k0 + lane : keyed - 1);
       // the last lane whose keys start at or before e (lanes without keys share their successor's start)
       int j = 0;
 #pragma unroll
@@ -254,7 +257,7 @@ __global__ void __launch_bounds__(256) k_splat_keys(int64_t n, const uint32_t* _
       }
       const uint32_t oj = __shfl_sync(0xFFFFFFFFu, o, j), ij = __shfl_sync(0xFFFFFFFFu, i, j);
       const int fj = __shfl_sync(0xFFFFFFFFu, first, j), wj = __shfl_sync(0xFFFFFFFFu, wide, j);
-      if (e < end) {
+      if (live) {
         const int k = (int)(e - oj), row = k / wj;
         keys[e] = (K)(fj + row * tiles_x + (k - row * wj));
         vals[e] = ij;
@@ -362,18 +365,20 @@ __global__ void __launch_bounds__(32) k_render(const uint2* __restrict__ ranges,
   __shared__ float4 s0[RSTAGE], s1[RSTAGE], s2[RSTAGE], s3[RSTAGE];
   const int lane = threadIdx.x;
   int tile = blockIdx.x, slot = -1;
-  uint2 rg;
+  uint32_t first, len;  // of the list, or of its segment
   if (tile < tiles) {
-    rg = ranges[tile];
-    if (rg.y - rg.x > RSEG) return;
+    const uint2 rg = ranges[tile];
+    first = rg.x;
+    len = rg.y - rg.x;
+    if (len > RSEG) return;
   } else {
     slot = tile - tiles;
     if (slot >= (int)*n_segs) return;
     const Segment s = segs[slot];
     tile = (int)s.tile;
-    rg = ranges[tile];
-    rg.x += s.seg * RSEG;
-    rg.y = min(rg.y, rg.x + RSEG);
+    const uint2 rg = ranges[tile];
+    first = rg.x + s.seg * RSEG;
+    len = min(rg.y - first, (uint32_t)RSEG);
   }
   const int tx = tile % tiles_x, ty = tile / tiles_x;
   const int px = tx * RTILE + (lane & 15), py = ty * RTILE + (lane >> 4);  // rows py, py + 2, .. py + 14
@@ -385,22 +390,24 @@ __global__ void __launch_bounds__(32) k_render(const uint2* __restrict__ ranges,
     T[j] = make_float2(1.0f, 1.0f);
     r[j] = g[j] = b[j] = make_float2(0.0f, 0.0f);
   }
-  // entry indices two stages ahead, records one
-  uint32_t id = rg.x + lane < rg.y ? vals[rg.x + lane] : 0u;
+  // entry indices two stages ahead, records one; steps count from the list's first entry (an entry's number plus a step
+  // may be past 2^32)
+  const uint32_t* list = vals + first;
+  uint32_t id = lane < len ? list[lane] : 0u;
   float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f), n1 = n0;
   float n2 = 0.f;
-  if (rg.x + lane < rg.y) { const float4* p = rec + 3 * (int64_t)id; n0 = p[0]; n1 = p[1]; n2 = p[2].x; }
-  id = rg.x + RSTAGE + lane < rg.y ? vals[rg.x + RSTAGE + lane] : 0u;
-  for (uint32_t e0 = rg.x; e0 < rg.y; e0 += RSTAGE) {
+  if (lane < len) { const float4* p = rec + 3 * (int64_t)id; n0 = p[0]; n1 = p[1]; n2 = p[2].x; }
+  id = RSTAGE + lane < len ? list[RSTAGE + lane] : 0u;
+  for (uint32_t k0 = 0; k0 < len; k0 += RSTAGE) {
     __syncwarp();
     s0[lane] = make_float4(n0.x, n0.z, n0.w, 0.f);
     s1[lane] = make_float4(-n0.y, -n0.y, n1.x, n1.x);
     s2[lane] = make_float4(n1.y, n1.y, n1.z, n1.z);
     s3[lane] = make_float4(n1.w, n1.w, n2, n2);
     __syncwarp();
-    if (e0 + RSTAGE + lane < rg.y) { const float4* p = rec + 3 * (int64_t)id; n0 = p[0]; n1 = p[1]; n2 = p[2].x; }
-    if (e0 + 2 * RSTAGE + lane < rg.y) id = vals[e0 + 2 * RSTAGE + lane];
-    const int m = (int)min((uint32_t)RSTAGE, rg.y - e0);
+    if (k0 + RSTAGE + lane < len) { const float4* p = rec + 3 * (int64_t)id; n0 = p[0]; n1 = p[1]; n2 = p[2].x; }
+    if (k0 + 2 * RSTAGE + lane < len) id = list[k0 + 2 * RSTAGE + lane];
+    const int m = (int)min((uint32_t)RSTAGE, len - k0);
 #pragma unroll 8
     for (int k = 0; k < m; k++) {
       const float4 a = s0[k], c = s1[k], d = s2[k], h = s3[k];
