@@ -29,6 +29,10 @@
  *  - There is no CPU fallback: without a usable GB300 every call returns
  *    GSC_ERR_UNSUPPORTED (except the host-only calls: gsc_server_simulate and the
  *    checkpoint file calls on host buffers).
+ *  - Calls of one context on different streams run independently, but for the plan: its two halves
+ *    run beside one another on the caller's stream and one of the context's four side streams, taken in turn,
+ *    so a plan may wait for the fourth plan before it on another stream. (On a stream of other than
+ *    the default priority, and under capture, all of a plan is on the caller's stream.)
  *  - A context serves one host thread at a time (it holds a pinned staging buffer and the
  *    kernel timers); use one context per thread, as the request loop does per worker. The
  *    request loop's own calls (gsc_server_*) may be made from any thread.

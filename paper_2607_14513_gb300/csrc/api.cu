@@ -260,9 +260,11 @@ extern "C" gsc_status gsc_ctx_create(gsc_ctx** out, int device) { return ctx_new
 static void ctx_free(gsc_ctx* c) {
   if (c->d_status) cudaFree(c->d_status);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
-  if (c->side_join) cudaEventDestroy(c->side_join);
-  if (c->side_fork) cudaEventDestroy(c->side_fork);
-  if (c->side) cudaStreamDestroy(c->side);
+  for (gsc_side& s : c->side) {
+    if (s.join) cudaEventDestroy(s.join);
+    if (s.fork) cudaEventDestroy(s.fork);
+    if (s.st) cudaStreamDestroy(s.st);
+  }
   free(c);
 }
 
@@ -287,9 +289,11 @@ gsc_status ctx_new(int device, bool init_tables, gsc_ctx** out) {
   if (e == cudaSuccess) { c->d_diag = c->d_status + 1; e = cudaMemset(c->d_status, 0, 2 * sizeof(int)); }
   if (e == cudaSuccess) e = cudaMallocHost(&c->h_pinned, PINNED_BYTES);
   c->h_pinned_bytes = PINNED_BYTES;
-  if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->side_fork, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&c->side_join, cudaEventDisableTiming);
+  for (gsc_side& s : c->side) {
+    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s.st, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&s.join, cudaEventDisableTiming);
+  }
   if (init_tables) {
     if (e == cudaSuccess) e = bc1_init_tables();
     if (e == cudaSuccess) e = bc7_init_tables();

@@ -20,6 +20,13 @@ struct gsc_tex_slot {
   int64_t nblk;
 };
 
+// A plan's second stream and the events that tie it to the caller's.
+struct gsc_side {
+  cudaStream_t st;
+  cudaEvent_t fork, join;
+};
+#define GSC_SIDES 4
+
 struct gsc_ctx {
   int device;
   gsc_tex_slot tex[2];        // texture path: [0] BC1, [1] BC7, kept between calls
@@ -35,8 +42,8 @@ struct gsc_ctx {
   int* d_diag;          // where it happened (kernel-defined)
   void* h_pinned;       // small pinned host buffer for table read-back
   size_t h_pinned_bytes;
-  cudaStream_t side;    // for the half of a plan that runs beside the other
-  cudaEvent_t side_fork, side_join;
+  gsc_side side[GSC_SIDES];  // for the half of a plan that runs beside the other; plans take them in turn
+  unsigned side_turn;
 };
 
 #define GSC_CUDA(call)                                   \
