@@ -173,16 +173,22 @@ __global__ void k_finish_perm(const uint32_t* __restrict__ vals, int64_t n, int6
 
 // ---- the whole-scene plan -----------------------------------------------------------------------
 // Scales. Small scenes (up to PLAN_SMALL): one CTA per coefficient holds all its magnitudes in shared memory and
-// selects the rank by four 8-bit digits. Larger ones: a stratified sample of 4096 Gaussians brackets each
-// coefficient's rank (six standard deviations of the sample's rank either way, under 1% of the values), one read of
-// the scene counts what lies below and at the bracket's ends and collects what lies inside, and one CTA per
-// coefficient selects among those. The four full reads that a plain radix selection takes (576 MB each at 3M
-// Gaussians, every value an atomic in shared memory) were 720 of 1570 us; the bracketed one is 40 + 138 + 57 us, its
-// read at 61% of the copy bandwidth. Where
-// the rank is outside its bracket or the inside overflows its buffer (a sample that does not stand for the scene),
-// that CTA selects over the whole scene: the result is the exact order statistic either way.
+// selects the rank, ten bits at a time. Larger ones: a stratified sample of 4,096 Gaussians brackets each
+// coefficient's rank (six standard deviations of the sample's rank either way), one read of the scene counts what lies
+// below and at the bracket's ends and collects what lies inside, and one CTA per coefficient selects among those. The
+// four full reads that a plain radix selection takes (576 MB each at 3M Gaussians, every value an atomic in shared
+// memory) were 720 of 1570 us; the bracketed one is 30 + 122 + 64 us, its read at 69% of the copy bandwidth.
+// At 995 permille 0.9% of the values lie inside. Towards the middle of the distribution it would be up to 5.5%, more
+// than there is room for (n / 8 of a coefficient's 3 n): where it is more than SEL_WIDE the sample is three times as
+// large, and 3.2% lie inside at 500 permille (71 + 152 + 190 us; 11.9 ms in all when it did not fit). The line: 3M
+// Gaussians at 970 permille (2.0%) take 467 us with the large sample, 479 with the small one, 100,000 without the
+// sort 111 and 77.
+// Where the rank is outside its bracket or the inside overflows its buffer all the same (a sample that does not stand
+// for the scene), that CTA selects over the whole scene: the result is the exact order statistic either way.
 #define PLAN_SMALL 8192
 #define SEL_SAMPLE 4096
+#define SEL_SAMPLE_WIDE 12288
+#define SEL_WIDE 0.02
 #define SEL_THREADS 1024
 
 struct SelBracket {
@@ -250,26 +256,31 @@ __device__ __forceinline__ float scale_of(uint32_t bits) {
   return s == 0.0f ? 1.0f : s;
 }
 
-// CTAs 2 k and 2 k + 1: the low and the high end of coefficient k's bracket from the sample, and cleared counters
+// half the bracket's width in ranks of a sample of m values, around quantile q
+__host__ __device__ __forceinline__ double sel_half(double q, int m) { return 6.0 * sqrt((double)m * q * (1.0 - q)) + 8.0; }
+
+// CTAs 2 k and 2 k + 1: the low and the high end of coefficient k's bracket from a sample of SAMPLE Gaussians, and cleared
+// counters
+template <int SAMPLE>
 __global__ void __launch_bounds__(SEL_THREADS) k_sel_sample(const float* __restrict__ sh, int64_t n, unsigned long long rank,
                                                            SelBracket* __restrict__ S) {
-  extern __shared__ uint32_t v[];  // 3 * SEL_SAMPLE
+  extern __shared__ uint32_t v[];  // 3 * SAMPLE
   __shared__ uint32_t hist[1024], pick[34];
-  const int k = blockIdx.x >> 1, m = 3 * SEL_SAMPLE;
+  const int k = blockIdx.x >> 1, m = 3 * SAMPLE;
   const bool low = (blockIdx.x & 1) == 0;
-#pragma unroll
+#pragma unroll 12
   for (int j = 0; j < m / SEL_THREADS; j++) {
-    // one Gaussian of each of the 4096 equal strata, at a place drawn by a hash
+    // one Gaussian of each of SAMPLE equal strata, at a place drawn by a hash
     const int i = j * SEL_THREADS + threadIdx.x;
     const uint64_t g = (uint64_t)(i / 3);
     uint64_t h = (g + 1) * 0x9E3779B97F4A7C15ull;
     h = (h ^ (h >> 29)) * 0xBF58476D1CE4E5B9ull;
-    const int64_t at = (int64_t)((g * (uint64_t)n + (h >> 16) % (uint64_t)n) / SEL_SAMPLE);
+    const int64_t at = (int64_t)((g * (uint64_t)n + (h >> 16) % (uint64_t)n) / SAMPLE);
     v[i] = magnitude(__ldg(sh + at * 48 + 3 * k + i % 3));
   }
   __syncthreads();
   const double q = ((double)rank + 0.5) / (3.0 * (double)n), mid = q * m;
-  const double wide = 6.0 * sqrt((double)m * q * (1.0 - q)) + 8.0;
+  const double wide = sel_half(q, m);
   const int64_t a = (int64_t)floor(mid - wide), b = (int64_t)ceil(mid + wide);
   auto get = [&](int64_t i) { return v[i]; };
   if (low) {
@@ -286,15 +297,18 @@ __global__ void __launch_bounds__(SEL_THREADS) k_sel_sample(const float* __restr
 }
 
 // One read of the scene. The grid's threads are a multiple of 12, so a thread's float4s always hold the same four
-// places of the 48 and its brackets stay in registers; what lies inside (under 1%) goes through a buffer per CTA.
+// places of the 48 and its brackets stay in registers; what lies inside goes through a buffer per CTA, which is written
+// out every `rounds` rounds of four loads (a value of a full buffer takes a global addition of its own: the selection
+// at 900 permille and 12M Gaussians took 9.2 ms, against 1.0 ms). Four CTAs per SM: 3M Gaussians 122 us, with three
+// (76 registers) 138.
 #define SEL_KEEP 256
 struct SelCand {
   uint32_t* half[2];  // of coefficients 0-7 and 8-15
   uint32_t cap;       // values of one coefficient
   __device__ __forceinline__ uint32_t* of(int k) const { return half[k >> 3] + (int64_t)(k & 7) * cap; }
 };
-__global__ void __launch_bounds__(256) k_sel_scan(const float4* __restrict__ sh4, int64_t n4, SelBracket* __restrict__ S,
-                                                  SelCand cand) {
+__global__ void __launch_bounds__(256, 4) k_sel_scan(const float4* __restrict__ sh4, int64_t n4, int rounds,
+                                                  SelBracket* __restrict__ S, SelCand cand) {
   __shared__ uint32_t s_buf[GSC_SH][SEL_KEEP];
   __shared__ uint32_t s_n[GSC_SH], s_at[GSC_SH];
   __shared__ uint32_t s_cnt[3][GSC_SH];
@@ -328,15 +342,36 @@ __global__ void __launch_bounds__(256) k_sel_scan(const float4* __restrict__ sh4
       }
     }
   };
+  const int64_t full = n4 / (4 * step);  // rounds that every thread of the grid has
   int64_t i = i0;
-  for (; i + 3 * step < n4; i += 4 * step) {
-    const float4 a = __ldg(sh4 + i), b = __ldg(sh4 + i + step), c = __ldg(sh4 + i + 2 * step), d = __ldg(sh4 + i + 3 * step);
-    count(a);
-    count(b);
-    count(c);
-    count(d);
+  for (int64_t r = 0;;) {
+    const int64_t stop = min(full, r + rounds);
+    for (; r < stop; r++, i += 4 * step) {
+      const float4 a = __ldg(sh4 + i), b = __ldg(sh4 + i + step), c = __ldg(sh4 + i + 2 * step), d = __ldg(sh4 + i + 3 * step);
+      count(a);
+      count(b);
+      count(c);
+      count(d);
+    }
+    if (r == full)
+      for (; i < n4; i += step) count(__ldg(sh4 + i));
+    __syncthreads();
+    if (threadIdx.x < GSC_SH) {
+      const int k = threadIdx.x;
+      const uint32_t m = min(s_n[k], (uint32_t)SEL_KEEP);
+      s_n[k] = m;
+      s_at[k] = m ? atomicAdd(&S->inside[k], m) : 0u;
+    }
+    __syncthreads();
+    for (int x = threadIdx.x; x < GSC_SH * SEL_KEEP; x += 256) {
+      const int k = x / SEL_KEEP, j = x % SEL_KEEP;
+      if (j < (int)s_n[k] && s_at[k] + (uint32_t)j < cand.cap) cand.of(k)[s_at[k] + j] = s_buf[k][j];
+    }
+    if (r == full) break;
+    __syncthreads();
+    if (threadIdx.x < GSC_SH) s_n[threadIdx.x] = 0u;
+    __syncthreads();
   }
-  for (; i < n4; i += step) count(__ldg(sh4 + i));
 #pragma unroll
   for (int q = 0; q < 4; q++) {
     const int k = (j0 + q) / 3;
@@ -347,17 +382,9 @@ __global__ void __launch_bounds__(256) k_sel_scan(const float4* __restrict__ sh4
   __syncthreads();
   if (threadIdx.x < GSC_SH) {
     const int k = threadIdx.x;
-    const uint32_t m = min(s_n[k], (uint32_t)SEL_KEEP);
-    s_n[k] = m;
-    s_at[k] = m ? atomicAdd(&S->inside[k], m) : 0u;
     if (s_cnt[0][k]) atomicAdd(&S->below[k], (unsigned long long)s_cnt[0][k]);
     if (s_cnt[1][k]) atomicAdd(&S->at_lo[k], (unsigned long long)s_cnt[1][k]);
     if (s_cnt[2][k]) atomicAdd(&S->at_hi[k], (unsigned long long)s_cnt[2][k]);
-  }
-  __syncthreads();
-  for (int x = threadIdx.x; x < GSC_SH * SEL_KEEP; x += 256) {
-    const int k = x / SEL_KEEP, j = x % SEL_KEEP;
-    if (j < (int)s_n[k] && s_at[k] + (uint32_t)j < cand.cap) cand.of(k)[s_at[k] + j] = s_buf[k][j];
   }
 }
 
@@ -572,7 +599,9 @@ size_t plan_ws_bytes(int64_t n) { return carve_plan(nullptr, n).end + 256; }
 
 #define SMALL_SORT_BYTES (PLAN_SMALL * 6 + (SEL_THREADS / 32) * 1024)
 cudaError_t plan_init() {  // dynamic shared memory above 48 KB, once per device
-  cudaError_t e = cudaFuncSetAttribute(k_sel_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, 12 * SEL_SAMPLE);
+  cudaError_t e = cudaFuncSetAttribute(k_sel_sample<SEL_SAMPLE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 12 * SEL_SAMPLE);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_sel_sample<SEL_SAMPLE_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 12 * SEL_SAMPLE_WIDE);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_plan_small, cudaFuncAttributeMaxDynamicSharedMemorySize, 12 * PLAN_SMALL);
   return e;
 }
@@ -647,8 +676,17 @@ gsc_status plan_run(gsc_ctx* ctx, const float* pos, const float* sh, const gsc_p
     cand.cap = (uint32_t)(n / 8);
     const int64_t n4 = n * 12, want = ceil_div64(n4, 256 * 4), most = (int64_t)ctx->sm_count * 8;
     const int64_t g = (want < most ? want : most) / 3 * 3;
-    gsc_count_launch(); k_sel_sample<<<2 * GSC_SH, SEL_THREADS, 12 * SEL_SAMPLE, side.st>>>(sh, n, rank, w.sel);
-    gsc_count_launch(); k_sel_scan<<<(int)g, 256, 0, side.st>>>(reinterpret_cast<const float4*>(sh), n4, w.sel, cand);
+    // the bracket's share of the values, and how many rounds (256 values of a coefficient each) leave a third of the
+    // buffer to chance
+    const double q = ((double)rank + 0.5) / (3.0 * (double)n);
+    double share = 2.0 * sel_half(q, 3 * SEL_SAMPLE) / (3 * SEL_SAMPLE);
+    const bool wide = share > SEL_WIDE;
+    if (wide) share = 2.0 * sel_half(q, 3 * SEL_SAMPLE_WIDE) / (3 * SEL_SAMPLE_WIDE);
+    const int rounds = (int)(0.67 * SEL_KEEP / (256.0 * share)) + 1;
+    gsc_count_launch();
+    if (wide) k_sel_sample<SEL_SAMPLE_WIDE><<<2 * GSC_SH, SEL_THREADS, 12 * SEL_SAMPLE_WIDE, side.st>>>(sh, n, rank, w.sel);
+    else k_sel_sample<SEL_SAMPLE><<<2 * GSC_SH, SEL_THREADS, 12 * SEL_SAMPLE, side.st>>>(sh, n, rank, w.sel);
+    gsc_count_launch(); k_sel_scan<<<(int)g, 256, 0, side.st>>>(reinterpret_cast<const float4*>(sh), n4, rounds, w.sel, cand);
     gsc_count_launch(); k_sel_final<<<GSC_SH, SEL_THREADS, 0, side.st>>>(sh, n, rank, w.sel, cand, scales);
     GSC_CUDA(side.done());
   }
