@@ -647,7 +647,7 @@ gsc_status render_run(gsc_ctx* c, const DevTable& T, const uint8_t* d_blocks, co
       GSC_CUDA(cudaGetLastError());
     }
     // visible Gaussians nearest first (stable: equal depths in index order), their counts in that order
-    uint32_t *dk, *dv;  // four passes: the result is back in dval, which the pair buffers do not touch
+    uint32_t *dk, *dv;  // four passes, or none: the result is in dval, which the pair buffers do not touch
     GSC_CUDA(radix_sort<uint32_t>(w.dkey, w.dkey2, w.dval, w.vals2, n, 32, true, false, w.radix_state, st, &dk, &dv));
     gsc_count_launch();
     k_gather_counts<<<grid_of(n), 256, 0, st>>>(n, w.dval, w.count, w.count_sorted);
