@@ -177,11 +177,12 @@ __global__ void __launch_bounds__(256) k_rs_rows(uint32_t* __restrict__ counts, 
   if (t == 0) total[blockIdx.x] = carry;
 }
 
-// vin = nullptr: values are the input positions; kout = nullptr: the sorted keys are not wanted. mask: the pass's digit
-// as it was counted; BITS, at least as many, is the number of ballots that tell two digits apart.
+// vin = nullptr: values are the input positions; kout = nullptr: the sorted keys are not wanted. digit_mask: the pass's
+// digit as it was counted. From 5 bits on it is known from BITS (with the mask in a register 30M pairs of 16-bit keys
+// take 154 us instead of 149).
 template <class K, int BITS>
 __global__ void __launch_bounds__(RS_THREADS, 3)
-    k_rs_scatter(const K* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t n, int shift, uint32_t mask,
+    k_rs_scatter(const K* __restrict__ kin, const uint32_t* __restrict__ vin, int64_t n, int shift, uint32_t digit_mask,
                  const uint32_t* __restrict__ total, const uint32_t* __restrict__ counts, K* __restrict__ kout,
                  uint32_t* __restrict__ vout) {
   __shared__ K s_key[RS_TILE];
@@ -189,6 +190,7 @@ __global__ void __launch_bounds__(RS_THREADS, 3)
   __shared__ uint32_t s_cnt[RS_WARPS][256];
   __shared__ uint32_t s_start[256], s_base[256];
   __shared__ uint64_t s_scan[8];
+  const uint32_t mask = BITS > 4 ? (1u << BITS) - 1u : digit_mask;
   const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   const int64_t base = (int64_t)blockIdx.x * RS_TILE;
   const int count = (int)min((int64_t)RS_TILE, n - base);
@@ -254,6 +256,7 @@ cudaError_t radix_sort(K* keys, K* keys2, uint32_t* vals, uint32_t* vals2, int64
     const uint32_t* vin = p == 0 && iota ? nullptr : vals;
     K* kout = p + 1 < passes || want_keys ? keys2 : nullptr;
     if (d.ballots == 4) k_rs_scatter<K, 4><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, d.shift, d.mask, total, counts, kout, vals2);
+    else if (d.ballots == 5) k_rs_scatter<K, 5><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, d.shift, d.mask, total, counts, kout, vals2);
     else if (d.ballots == 6) k_rs_scatter<K, 6><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, d.shift, d.mask, total, counts, kout, vals2);
     else if (d.ballots == 7) k_rs_scatter<K, 7><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, d.shift, d.mask, total, counts, kout, vals2);
     else k_rs_scatter<K, 8><<<nt, RS_THREADS, 0, st>>>(keys, vin, n, d.shift, d.mask, total, counts, kout, vals2);

@@ -7,7 +7,7 @@ struct SortDigit {
   int shift, bits;  // the pass sorts by bits shift .. shift + bits - 1 of the key
   uint32_t mask;    // of the digit, for every kernel of the pass: one that took more bits than were counted would find
                     // no counts for its digits, and write past the end
-  int ballots;      // the scatter's instantiation (4, 6, 7 or 8): at least bits
+  int ballots;      // the scatter's instantiation, 4 to 8: bits, but 4 for fewer
 };
 
 inline int sort_passes(int key_bits) { return (key_bits + 7) / 8; }
@@ -21,6 +21,6 @@ inline SortDigit sort_digit(int key_bits, int p) {
     d.bits = (key_bits - d.shift + passes - q - 1) / (passes - q);
   }
   d.mask = (1u << d.bits) - 1u;
-  d.ballots = d.bits <= 4 ? 4 : d.bits <= 6 ? 6 : d.bits;
+  d.ballots = d.bits < 4 ? 4 : d.bits;
   return d;
 }
