@@ -240,6 +240,7 @@ static cudaError_t launch_bc7(const float* sh, const int32_t* perm, const float*
   const size_t smem = warps * sizeof(Bc7Warp);
   uint4* to = reinterpret_cast<uint4*>(out);
   gsc_count_launch();
+  static_assert(BC7_WARPS * sizeof(Bc7Warp) <= 48 * 1024, "more needs a raised limit");
   if (few) k_bc7<8, BC7_WARPS><<<(int)grid, 32 * warps, smem, st>>>(sh, perm, scales, n_groups, tex, nblk, to, sse7, sse64);
   else if (many) k_bc7<32, BC7_WIDE><<<(int)grid, 32 * warps, smem, st>>>(sh, perm, scales, n_groups, tex, nblk, to, sse7, sse64);
   else k_bc7<32, BC7_WARPS><<<(int)grid, 32 * warps, smem, st>>>(sh, perm, scales, n_groups, tex, nblk, to, sse7, sse64);
@@ -247,10 +248,8 @@ static cudaError_t launch_bc7(const float* sh, const int32_t* perm, const float*
 }
 
 cudaError_t bc7_init_kernels() {  // dynamic shared memory above 48 KB, once per device
-  cudaError_t e = cudaFuncSetAttribute(k_bc7<32, BC7_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)(BC7_WIDE * sizeof(Bc7Warp)));
-  return e == cudaSuccess ? cudaFuncSetAttribute(k_bc7<8, BC7_WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)(BC7_WARPS * sizeof(Bc7Warp))) : e;
+  return cudaFuncSetAttribute(k_bc7<32, BC7_WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)(BC7_WIDE * sizeof(Bc7Warp)));
 }
 
 cudaError_t launch_bc7_groups(const float* sh, const int32_t* perm, const float* scales, int64_t n_groups,
