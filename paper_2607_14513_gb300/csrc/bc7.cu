@@ -153,17 +153,18 @@ cudaError_t bc7_init_tables() {
 // quantisation tables, each stages and searches its own 32 blocks (two groups), and they go from phase to phase
 // together: bound by instruction issue and fetch, and warps in one phase run the same code. With barriers between the
 // phases and before the solve, and ten warps per CTA, 3M blocks of the scene with outliers take 28.7 ms, against 34.5 ms
-// with each of four warps at its own pace and 67.0 ms for the exhaustive search; 262,144 without outliers: 1.21, 1.39
-// and 6.95 ms. 20 warps per SM at most 102 registers; 24 at 80 and 16 at 128 were slower.
+// with each of four warps at its own pace and 67.0 ms for the exhaustive search; the call for 262,144 without outliers
+// 1.23, 1.40 and 6.98 ms. 20 warps per SM at most 102 registers; 24 at 80 and 16 at 128 were slower.
 #define BC7_WARPS 4
 // Up to this many blocks per SM a warp takes 8 blocks instead of 32: the chip has warps to spare and the time is
-// one warp's. Scene without outliers, 8 against 32 blocks per warp, each at its own pace: 4,096 blocks 187 against 265 us,
-// 10,000 209 against 268 us, 20,000 294 against 291 us, 40,000 521 against 335 us.
+// one warp's. Scene without outliers, 8 against 32 blocks per warp: 1,000 blocks 122 against 194 us, 4,096 138 against
+// 222, 10,000 157 against 226, 17,000 205 against 229, 20,000 239 and 239, 40,000 439 against 291.
 #define BC7_FEW 112
 #define BC7_MIN_BLOCKS 5
 // Above this many blocks per SM a CTA has ten warps instead of four: more warps share their phase's code, but a CTA of
-// 320 blocks leaves a larger part of the last wave idle. Ten against four: 120,000 blocks 694 against 673 us, 262,144
-// 1252 against 1279 us, the scene of 3M 31.1 against 34.3 ms; twenty: 120,000 801, 262,144 1200 us, 3M 31.2 ms.
+// 320 blocks leaves a larger part of the last wave idle. The kernel with ten against four: 120,000 blocks 637 against
+// 614 us, 180,000 804 against 824, 262,144 1164 and 1164, the scene of 3M with outliers 28.7 against 29.9 ms; with
+// twenty 754, 777, 1141 us and 28.8 ms.
 #define BC7_MANY 1280
 #define BC7_WIDE 10
 

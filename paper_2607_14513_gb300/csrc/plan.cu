@@ -610,8 +610,8 @@ static int bits_for(uint64_t v) { int b = 0; while (v) { b++; v >>= 1; } return 
 
 // The selection of the scales and the spatial order need nothing of each other, and neither fills the chip (the one
 // waits for the scene's bytes, or runs 16 CTAs; the other's passes are short): the selection goes to one of the
-// context's side streams. 3M Gaussians: the plan takes 441 us, against 545 us on one stream; 20,000: 114 against
-// 171 us. Plans take the side streams in turn, so that plans on up to four streams of a context (the batched form's
+// context's side streams. 3M Gaussians: the plan takes 460 us, against 547 us on one stream; 20,000: 147 against
+// 178 us. Plans take the side streams in turn, so that plans on up to four streams of a context (the batched form's
 // lanes) don't wait for one another: 64 scenes of 50,000 to 2M Gaussians planned on four streams 5.2 ms, against 6.3 ms
 // with one side stream for all and 5.8 ms with none. On a stream of another priority than the side streams' (the default)
 // all stays on that stream, and so it does under capture, so that a side stream is never part of a graph that

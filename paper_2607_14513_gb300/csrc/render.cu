@@ -322,10 +322,11 @@ __device__ __forceinline__ float ex2(float x) {
 // parity l / 16, in four pairs for the two-lane multiply-adds. Every pixel's exponent comes from its own distance to the
 // centre: stepping from the first row to the others, one instruction less per pair, adds terms of hundreds that cancel
 // for a splat of a pixel's size (relative error of a weight up to 6e-5 at a variance of 0.3 px^2, against 2e-6 at most)
-// and saved 1% of the frame. Records are staged 32 at a time through shared memory, the next 32 loaded while these are
-// blended. Bound by the multiply-add pipe (a splat is 32 two-lane instructions of two cycles and 8 others per warp):
-// 2.2 ms for the 29M (Gaussian, tile) pairs of a 1080p frame of 3M Gaussians, against 4.5 ms with four warps per tile
-// and two pixels per thread, which issued 15 instructions per pixel and read every splat four times.
+// and took 2.23 instead of 2.27 ms. Records are staged 32 at a time through shared memory, the next 32 loaded while these
+// are blended. Bound by the multiply-add pipe (72% busy; a splat is 32 two-lane instructions of two cycles and 8 others
+// per warp): 2.27 ms for the 29M (Gaussian, tile) pairs of a 1080p frame of 3M Gaussians, against 4.3 ms with four warps
+// per tile and two pixels per thread, which issued 15 instructions per pixel and read every splat four times. 100
+// registers; capped for 20 or 24 warps per SM it takes 1 and 2% longer.
 //
 // Blending is associative: a run of splats takes (colour, T) to (colour + T C', T T') with the run's own C' and
 // T'. Lists longer than RSEG are cut into segments of RSEG, each a warp's job with its result in a slot, joined

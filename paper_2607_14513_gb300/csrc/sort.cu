@@ -5,7 +5,8 @@
 // pairs of 32-bit keys (one GB300, each kernel alone with cold caches), against 12 + 15 + 58 us with a three-kernel
 // scan and three CTA barriers per 32 items in the scatter. The scatter is bound by latency: with the values read only
 // after the keys had been placed, and half the items in flight, it took 33 us, and 30M pairs of 16-bit keys 246 us
-// against 149 us; four CTAs per SM instead of three take as long. No kernel waits for another CTA: chaining the tiles in
+// against 149 us; three CTAs per SM (80 registers; 60 bytes spilled with 32-bit keys, 124 with 64-bit ones, none with
+// 16-bit ones) were best with 32-bit keys, four take as long with 16-bit ones. No kernel waits for another CTA: chaining the tiles in
 // one kernel (decoupled look-back) took 41 us per pass with two resident CTAs per SM and 470 us with four, when
 // most of the machine polled. 32-bit keys where the caller's fit.
 #include "sort.cuh"
