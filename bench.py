@@ -731,7 +731,7 @@ def run_render(args, world, rank, local):
     achieved = evals * 20 / (blend_ms * 1e-3) / 1e12
     roofline = {"bound": "alu", "achieved": round(achieved, 3), "peak": round(peak, 2), "unit": "TFLOP/s",
                 "frac": round(achieved / peak, 4), "traffic": None,
-                "kernel": "k_render (per-tile front-to-back blending, one thread per pixel)",
+                "kernel": "k_render (per-tile front-to-back blending, a warp per tile, eight pixels per thread)",
                 "peak_source": "FP32 FMA peak from the SM count, 128 lanes/SM and the sampled SM clock",
                 "algorithmic": "256 pixels x %d (Gaussian, tile) pairs per frame (mean) x 20 flops" % (sum(pairs) // V)}
     stages = {"frame_ms": round(ms_step / V, 3), "render_call_ms": round(call_ms, 3),
